@@ -125,7 +125,8 @@ enum { MK_CLUSTER_AUTO = 0, MK_CLUSTER_OFF = 1, MK_CLUSTER_ON = 2 };
 int mk_ctx_set_cluster(mk_ctx *ctx, int mode);
 
 /* Test hook for the kernels' bounded waits (no paper counterpart).  Every
- * wait of the staged blind rotation (variant 6) for a key copy and of the
+ * wait of the staged blind rotation (variant 6) for a key copy, of the warp
+ * kernel (variant 2) for its matrix products and of the
  * tcgen05 product engine (MK_FORM_TC, variant 1) gives up after wait_ns of
  * global time (0: the default, 1 s); a kernel whose wait gave up stops its
  * work, lets its own copies and tensor-core operations finish, and returns
@@ -195,7 +196,8 @@ int mk_ctx_get_circuit_style(const mk_ctx *ctx, int *style);
 /* Blind-rotation kernel variants (same results, different register/occupancy
  * trade-offs): 0..MK_NUM_VARIANTS-1.  0-5: one CTA per gate, with different
  * digit polynomials per forward pass, register caps, twiddle placement and
- * elements per thread; 6: several gates per CTA sharing each CMux step's
+ * elements per thread (under MK_FORM_NTT2 at N = 1024 with bg_bit 8, 2 is the
+ * warp kernel: tcgen05 products for the first transform stages); 6: several gates per CTA sharing each CMux step's
  * bootstrapping-key entry, bulk-copied once into shared memory; 7, 8
  * (MK_FORM_NTT2): the two primes' transforms on separate warps, recombined
  * by CRT through shared memory (MK_FORM_NTT runs variant 2's kernel for 7

@@ -203,23 +203,25 @@ struct FieldDual {
 };
 
 // Layouts of an NTT-domain key polynomial (transform order), chosen so that
-// a thread holding EPT = 8 consecutive elements reads them with 16-byte loads
-// that are contiguous across the warp: coalesced in global memory and free of
-// bank conflicts in shared memory.
+// threads holding consecutive elements read them with 16-byte loads that are
+// coalesced in global memory and free of bank conflicts in shared memory.
 //  * 8-byte elements (MK_FORM_NTT): the 16-byte unit u (elements 2u, 2u + 1)
 //    is stored at unit position (u % 4) * (N / 8) + u / 4, so unit q of
 //    thread t's four is at q * (N / 8) + t.
 //  * two residues (MK_FORM_NTT2): two planes of N words (residues mod p1,
 //    then mod p2); in each plane the 16-byte unit u (elements 4u .. 4u + 3)
-//    is stored at (u % 2) * (N / 8) + u / 2, so unit r of thread t's two is
-//    at r * (N / 8) + t.  A kernel that works on one prime reads one plane.
+//    is stored at (u % 8) * (N / 32) + (u / 8 xor u % 8): a lane holding 32
+//    consecutive elements (eight units) reads unit v of each contiguous
+//    across the warp, and the exclusive or spreads the units of threads
+//    holding 8 or 4 elements over distinct shared-memory banks.  A kernel
+//    that works on one prime reads one plane.
 template <int LOGN>
 __host__ __device__ __forceinline__ int key_unit_pos(int u) {
     return (u & 3) * ((1 << LOGN) / 8) + (u >> 2);
 }
 template <int LOGN>
 __host__ __device__ __forceinline__ int plane_unit_pos(int u) {
-    return (u & 1) * ((1 << LOGN) / 8) + (u >> 1);
+    return (u & 7) * ((1 << LOGN) / 32) + ((u >> 3) ^ (u & 7));
 }
 
 template <bool SMEM>

@@ -368,8 +368,9 @@ struct mk_ctx {
         // twiddles: [2][N] of 8-byte (NTT) or 16-byte (NTT2) entries; FFT: one [3][N/2] table
         const size_t half = (form == MK_FORM_NTT2 ? 16 : (form == MK_FORM_FFT ? 0 : 8)) * (size_t)P.N;
         const void *split = form == MK_FORM_NTT2 ? (const unsigned char *)d_tw + 32 * (size_t)P.N : nullptr;
+        const void *warp = form == MK_FORM_NTT2 && P.N == 1024 ? (const unsigned char *)d_tw + 64 * (size_t)P.N : nullptr;
         return DeviceKeys{d_tw, (const unsigned char *)d_tw + half, d_bk, d_keyA, d_ks, d_tcws, tc_ws_gates, d_status,
-                          split};
+                          split, warp};
     }
 };
 

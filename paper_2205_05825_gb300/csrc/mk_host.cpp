@@ -190,6 +190,74 @@ int check_all_secret(mk_ctx *c) {
     return MK_OK;
 }
 
+// fp16 bits of an integer of magnitude at most 2048.
+uint16_t half_bits(int v) {
+    if (v == 0) return 0;
+    const uint16_t sign = v < 0 ? 0x8000 : 0;
+    uint32_t a = (uint32_t)(v < 0 ? -v : v);
+    int e = 0;
+    while ((a >> e) > 1) ++e;
+    return (uint16_t)(sign | ((15 + e) << 10) | ((a << 10 >> e) & 0x3FF));
+}
+
+// Tables of the warp kernel (layout in mk_bootstrap_warp.cuh): twiddles of
+// the last four stages by factor, of stage six by row of 32, of the first
+// five by heap index; the matrix operands: the planes of zeta_y^s, the powers
+// of the factors X^16 - zeta_y of X^1024 + 1 (zeta_2i = psi^bitrev(32 + i),
+// zeta_2i+1 = -zeta_2i), and the constants that start the sums.
+void warp_tables(const HostNtt32 &t1, const HostNtt32 &t2, unsigned char *out) {
+    std::memset(out, 0, kWarpTableBytes);
+    uint32_t *halves = reinterpret_cast<uint32_t *>(out);
+    uint32_t *rows = halves + 4 * (2 * 2 * 8 * 32);
+    uint32_t *cross = rows + 4 * (2 * 16);
+    uint16_t *start = reinterpret_cast<uint16_t *>(cross + 4 * (2 * 16));
+    uint16_t *planes = start + 8 * (2 * 128);
+    uint16_t *ones = planes + 8 * (3 * 4 * 256);
+    // offsets B of the first plane (prime_of in mk_bootstrap_warp.cuh) as 64 b1 + b0
+    const int b1[2] = {-256, -71}, b0[2] = {4, -7};
+    for (uint32_t pr = 0; pr < 2; ++pr) {
+        const HostNtt32 &t = pr ? t2 : t1;
+        const uint32_t p = t.p;
+        auto put = [p](uint32_t *dst, uint32_t w) {
+            dst[0] = w;
+            dst[1] = (uint32_t)(((uint64_t)w << 32) / p);
+        };
+        for (uint32_t x = 0; x < 32; ++x) {
+            put(rows + pr * 64 + 2 * x, t.psi_rev[32 + x]);
+            put(cross + pr * 64 + 2 * x, x ? t.psi_rev[x] : 0);
+        }
+        for (uint32_t y = 0; y < 64; ++y) {
+            uint32_t *lane = halves + ((pr * 2 + y / 32) * 8 * 32 + y % 32) * 4;  // unit u: 128 u words on
+            put(lane, 0);
+            for (uint32_t b = 1; b < 16; b <<= 1)
+                for (uint32_t i = 0; i < b; ++i)
+                    put(lane + (b + i) / 2 * 128 + ((b + i) & 1) * 2, t.psi_rev[64 * b + b * y + i]);
+            const uint32_t z = (y & 1) ? p - t.psi_rev[32 + y / 2] : t.psi_rev[32 + y / 2];
+            uint32_t pow[64] = {1};
+            for (uint32_t s = 1; s < 64; ++s) pow[s] = HostNtt32::mulm(pow[s - 1], z, p);
+            const uint32_t row = 64 * pr + y;
+            for (uint32_t k = 0; k < 64; ++k) {
+                const uint32_t i = k % 8, w = pow[2 * (k / 8) + 16 * (i / 2) + i % 2];
+                const int v = w > p / 2 ? (int)w - (int)p : (int)w;
+                const int v0 = ((v + 256) & 511) - 256, r = (v - v0) / 512, v1 = ((r + 256) & 511) - 256;
+                const int digit[3] = {v0, v1, (r - v1) / 512};
+                for (uint32_t pl = 0; pl < 3; ++pl)
+                    planes[(((pl * 4 + k / 16) * 2 + k / 8 % 2) * 128 + row) * 8 + i] = half_bits(digit[pl]);
+            }
+            for (uint32_t pl = 0; pl < 2; ++pl) {
+                start[(pl * 128 + row) * 8] = half_bits(3072);
+                start[(pl * 128 + row) * 8 + 1] = pl ? 0 : half_bits(b1[pr]);
+                start[(pl * 128 + row) * 8 + 2] = pl ? 0 : half_bits(b0[pr]);
+            }
+        }
+    }
+    for (uint32_t c = 0; c < 48; ++c) {
+        ones[8 * c] = half_bits(4096);
+        ones[8 * c + 1] = half_bits(64);
+        ones[8 * c + 2] = half_bits(1);
+    }
+}
+
 }  // namespace
 namespace mk {
 // Build the NTT-domain bootstrapping keys and upload everything the kernels read.
@@ -208,7 +276,8 @@ int ensure_device_keys(mk_ctx *c) {
     std::vector<uint64_t> h_bk(bk_entries * N), h_keyA(keyA_entries * N);
     // The largest twiddle tables of the forms: NTT2's [2][N] uint4 plus the
     // per-prime tables [2 directions][2 primes][N] uint2 of the split kernel.
-    std::vector<unsigned char> h_tw(4 * (size_t)N * 16);
+    // After them, at N = 1024, the tables of the warp kernel.
+    std::vector<unsigned char> h_tw(4 * (size_t)N * 16 + (N == 1024 ? kWarpTableBytes : 0));
     // src polynomial of BK entry e and of keyA entry r (negated for the CRS)
     auto bk_src = [&](size_t e) {
         const uint32_t i = (uint32_t)(e / ((size_t)n * 3 * d));
@@ -272,6 +341,7 @@ int ensure_device_keys(mk_ctx *c) {
             sp[2 * (2 * (size_t)N + m)] = i1, sp[2 * (2 * (size_t)N + m) + 1] = comp(i1, kP1);
             sp[2 * (3 * (size_t)N + m)] = i2, sp[2 * (3 * (size_t)N + m) + 1] = comp(i2, kP2);
         }
+        if (N == 1024) warp_tables(c->ntt_p1, c->ntt_p2, h_tw.data() + 4 * (size_t)N * 16);
         auto dual = [&](const uint32_t *src, uint64_t *dst, bool negate) {
             std::vector<uint32_t> r1(N), r2(N);
             c->ntt_p1.to_device(src, r1.data(), negate);
@@ -290,7 +360,7 @@ int ensure_device_keys(mk_ctx *c) {
         //  NTT: 16-byte unit u (elements 2u, 2u + 1) goes to (u % 4) * (N / 8) + u / 4.
         //  NTT2: the {r1, r2} pairs split into a plane of r1 and a plane of r2;
         //  in each, the 16-byte unit u (elements 4u .. 4u + 3) goes to
-        //  (u % 2) * (N / 8) + u / 2.
+        //  (u % 8) * (N / 32) + (u / 8 xor u % 8).
         const bool planes = c->form == MK_FORM_NTT2;
         auto interleave = [N, planes](uint64_t *poly, std::vector<uint64_t> &tmp) {
             tmp.assign(poly, poly + N);
@@ -300,7 +370,7 @@ int ensure_device_keys(mk_ctx *c) {
                 uint32_t *dst = reinterpret_cast<uint32_t *>(poly);
                 for (uint32_t pl = 0; pl < 2; ++pl)
                     for (uint32_t u = 0; u < N / 4; ++u) {
-                        const uint32_t pos = (u & 1) * stride + (u >> 1);
+                        const uint32_t pos = (u & 7) * (N / 32) + ((u >> 3) ^ (u & 7));
                         for (uint32_t e = 0; e < 4; ++e) dst[pl * N + 4 * pos + e] = src[2 * (4 * u + e) + pl];
                     }
                 return;
@@ -907,6 +977,8 @@ int mk_sync(mk_ctx *c) {
             MK_CUDA(c, cudaMemset(c->d_status, 0, sizeof(st)));
             if (st & kStatusStaged)
                 return fail(c, MK_ETIMEOUT, "a bounded wait of the staged blind rotation for a key copy gave up");
+            if (st & kStatusWarp)
+                return fail(c, MK_ETIMEOUT, "a matrix product of the blind rotation did not complete in time");
             if (st & kStatusCluster)
                 return fail(c, MK_ETIMEOUT, "a bounded wait of the cluster blind rotation for a key copy gave up");
             return fail(c, MK_ETIMEOUT, "the persistent operator launch made no progress within its bound");

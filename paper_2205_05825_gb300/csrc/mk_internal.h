@@ -47,15 +47,22 @@ struct DeviceKeys {
     void *tc_ws;
     uint32_t tc_ws_gates;
     // The context's status word (device): a kernel whose bounded wait ran out
-    // sets its bit (kStatusStaged, kStatusNetlist, kStatusCluster); mk_sync reports it as
+    // sets its bit (kStatusStaged, kStatusNetlist, kStatusCluster, kStatusWarp); mk_sync reports it as
     // MK_ETIMEOUT and clears it.
     uint32_t *status;
     // MK_FORM_NTT2: per-prime twiddles [2 directions][2 primes][N] uint2
     // {w, w'} for the split-prime kernel (nullptr for the other forms).
     const void *tw_split;
+    // MK_FORM_NTT2 at N = 1024: the warp kernel's tables (kWarpTableBytes,
+    // layout in mk_bootstrap_warp.cuh); nullptr otherwise.
+    const void *tw_warp;
 };
 
-constexpr uint32_t kStatusStaged = 1u, kStatusNetlist = 2u, kStatusCluster = 4u;
+// Tables of the warp kernel: twiddles by factor and by stage, matrix operands.
+constexpr size_t kWarpTableBytes = 16 * (2 * 2 * 8 * 32 + 2 * 16 + 2 * 16 + 2 * 128 + 3 * 4 * 256 + 2 * 48);
+constexpr size_t kWarpSmemMax = 227 * 1024;
+
+constexpr uint32_t kStatusStaged = 1u, kStatusNetlist = 2u, kStatusCluster = 4u, kStatusWarp = 8u;
 
 struct LaunchShape {
     uint32_t n, N, logN, k, d, bg_bit, ks_bit, t;
@@ -101,7 +108,9 @@ cudaError_t launch_blind_rotate_ntt(const LaunchShape &S, const DeviceKeys &K, c
 // (mk_bootstrap_staged.cuh: G gates per CTA share each step's key entry,
 // bulk-copied into shared memory once); 2 is the split-prime kernel
 // (mk_bootstrap_split.cuh, MK_FORM_NTT2: one half of a gate's threads per
-// prime; MK_FORM_NTT runs variant 2's kernel for these numbers).  All give
+// prime; MK_FORM_NTT runs variant 2's kernel for these numbers).  Under
+// MK_FORM_NTT2 variant 2 runs the warp kernel (mk_bootstrap_warp.cuh) on the
+// shapes it supports.  All give
 // identical results.
 constexpr int kNumVariants = 9;
 constexpr int kVariantNpf[kNumVariants] = {3, 1, 3, 3, 3, 3, 3, 3, 3};
@@ -132,6 +141,14 @@ MK_DECLARE_BOOTSTRAP_F(10, 0)
 MK_DECLARE_BOOTSTRAP_F(10, 1)
 MK_DECLARE_BOOTSTRAP(8, 2, 0)
 MK_DECLARE_BOOTSTRAP(10, 2, 0)
+
+// The warp-per-prime kernel (mk_brw.cu): the two-prime form at N = 1024,
+// d = 3, bg_bit = 8.  Same arguments as the launchers above.
+bool warp_form_supported(const LaunchShape &S);
+cudaError_t launch_bootstrap_warp(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
+                                  const uint32_t *ct_a, const uint32_t *ct_b, const uint32_t *abar_in,
+                                  int64_t max_steps, uint32_t *ext, uint32_t *acc_out, uint32_t count,
+                                  cudaStream_t st);
 
 // Cluster (latency) form of the NTT blind rotation, one translation unit per
 // (ring dimension, field): mk_brc.cu built with -DMK_LOGN -DMK_FIELD.  Same
