@@ -34,16 +34,19 @@
 //    digits: eight coefficients of a lane are one 16-byte unit of the matrix
 //    operand, so v's digits need no further exchange.
 //  The four warps meet at a 128-thread barrier; gates of a CTA run
-//  independently of each other, so one gate's matrix products run under the
-//  others' butterflies.
+//  independently of each other.  A slot's matrix products are started as soon
+//  as the one before it has left TMEM, so they run under its butterflies; the
+//  first group of a slot's key words is loaded before them (two groups ahead
+//  measured slower: it spills).
 //
 // (The same matrix product by warp-level mma.sync gave 18.0 k clocks per CMux
 // step of a gate: on this chip it competes with the integer multiplies for
 // the register file, and its fragments need a transposition.)
 //
-// Measured (GB300, whole blind rotation): 4096 gates at k = 2 347 -> 244 ms,
-// 1001 at k = 4 308 -> 208 ms, 96 at k = 8 333 -> 159 ms, 152 at k = 2 (one gate
-// per SM) 31 -> 17.4 ms.  Per CMux step and gate 23.7 -> 16.7 k clocks of an SM.
+// Measured (GB300, whole blind rotation): 4096 gates at k = 2 347 -> 224 ms,
+// 1001 at k = 4 308 -> 192 ms, 96 at k = 8 333 -> 146 ms, 152 at k = 2 (one gate
+// per SM) 31 -> 15.0 ms.  Per CMux step and gate 23.7 -> 15.4 k clocks of an SM;
+// the multiply pipe's own share is 10 k.
 //
 // A CTA holds G gates (4 G warps) and the tables once; the grid is at most one
 // CTA per SM and walks the gates with stride G * gridDim.
@@ -343,6 +346,18 @@ __device__ __forceinline__ void half_inverse_stage(uint32_t (&y)[16], const uint
     }
 }
 
+// CRT (Garner) of residues x1 mod p1, x2 mod p2, each below 4 p, to the exact
+// integer mod 2^32: t p1 + x1 with t = (x2 - x1) / p1 mod p2 taken in
+// (-p2/2, p2/2).  x1 need not be canonical (t follows it), and the integers
+// are below 2^52.8 in magnitude against p1 p2 / 2 > 2^54.9, so t is never near
+// its boundary.  t comes centred from a product that is offset by h =
+// (p2 - 1) / 2: the operand is offset by h p1 mod p2.
+constexpr uint32_t CRT_H = (P2 - 1) / 2, CRT_HP1 = (uint32_t)((uint64_t)CRT_H * P1 % P2);
+__device__ __forceinline__ uint32_t crt_centred(uint32_t x1, uint32_t x2) {
+    const uint32_t t = shoup_k(x2 - x1 + (5 * P2 + CRT_HP1), CRT_C, CRT_CP, P2);
+    return min(t, t - P2) * P1 + (x1 - CRT_H * P1);
+}
+
 // Inverse transform of this lane's half row of residues (below 4 p), and
 // recombination: z[i] is the integer (mod 2^32) of coefficient c + 16 (i % 2) +
 // 32 (a + 8 (i / 2)), c = lane % 16, a = 2 warp + lane / 16.
@@ -453,15 +468,13 @@ __device__ __forceinline__ void inverse_crt(uint32_t (&y)[16], uint32_t (&z)[8],
             inv_bf(v[1], v[3], S1.z, S1.w, 2 * p, p);
             v[0] = min(v[0], v[0] - 8 * p);
             v[0] = min(v[0], v[0] - 4 * p);
-            v[0] = min(v[0], v[0] - 2 * p);
-            v[1] = min(v[1], v[1] - 2 * p);
 #pragma unroll
             for (int b = 0; b < 4; ++b) res[pr][g + 2 * b] = v[b];
         }
     }
     quad_sync(bar);  // every read of the exchange buffer is done
 #pragma unroll
-    for (int c = 0; c < 8; ++c) z[c] = FieldDual::to_u32(make_uint2(res[0][c], res[1][c]));
+    for (int c = 0; c < 8; ++c) z[c] = crt_centred(res[0][c], res[1][c]);
 }
 
 // x0 k0 + x1 k1 + x2 k2 (Montgomery keys), below 3.6 p for x below 13.6 p.
@@ -472,6 +485,19 @@ __device__ __forceinline__ uint32_t mac3_redc(uint32_t x0, uint32_t x1, uint32_t
     t += (uint64_t)x2 * k2;
     const uint32_t h = __umulhi((uint32_t)t * q.pinv, q.p);
     return (uint32_t)(t >> 32) - h + q.p;
+}
+
+// Units `low` of the lane's factor in three polynomials of each of two keys.
+__device__ __forceinline__ void load_keys(uint4 (&key)[6], const uint4 *k1, const uint4 *k2, uint32_t low,
+                                          uint32_t eighth) {
+    const uint32_t pos = low * 32 + (eighth ^ low);
+#pragma unroll
+    for (int l = 0; l < 6; ++l) {
+        const uint4 *src = (l < 3 ? k1 : k2) + (l % 3) * 512 + pos;
+        asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(key[l].x), "=r"(key[l].y), "=r"(key[l].z), "=r"(key[l].w)
+                     : "l"(src));
+    }
 }
 
 __device__ __forceinline__ uint32_t word_of(const uint4 &a, int h) {
@@ -559,129 +585,144 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
             for (uint32_t x = N + t128; x < (uint32_t)(k + 1) * N; x += 128) acc[x] = 0;
         }
         quad_sync(bar);
-        int step = 0;
-#pragma unroll 1
-        for (int i = 1; i <= k && step < limit; ++i) {
-#pragma unroll 1
-            for (int j = 0; j < n && step < limit; ++j, ++step) {
-                const uint32_t e = abar[step];
-                if (e == 0) continue;  // X^0 - 1 = 0: every digit is 0, the product adds nothing
-                const uint4 *bk = bk_all + (size_t)step * 9 * POLY + pr * (POLY / 2);
-                uint32_t V[16];
+        // The digits of (X^-e - 1) ACC_jj, and one thread's issue of their products once all are stored.
+        auto cut_digits = [&](int jj, uint32_t e) {
+            const uint32_t *ap = acc + jj * N;
+            uint32_t w[8];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) V[c] = 0;
-                // Slots 0..k: accumulator polynomials, the other parties' first, then 0, then i;
-                // slot k + 1: the digits of v.
+            for (int i8 = 0; i8 < 8; ++i8) {
+                const uint32_t r = m0 + 16 * (i8 & 1) + 256 * (i8 >> 1) + e;
+                const uint32_t a = ap[acc_pos(r & (N - 1))];
+                const uint32_t neg = (uint32_t)((int32_t)(r << 21) >> 31);  // bit 10 of r: -1
+                w[i8] = (a ^ neg) - neg - ap[(sw0 ^ (16 * (i8 & 1))) + 256 * (i8 >> 1)] + gad.offset;
+            }
+            store_digits(unit, w);
+        };
+        auto start_products = [&]() {
+            st_fence_proxy_async();
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+            quad_sync(bar);
+            if (warp == 0 && lane == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                issue_products(tmem, start_s, planes_s, ones_s, digits_s, mbar);
+            }
+            __syncwarp();
+        };
+        // Slots 0..k of a step: accumulator polynomials, the other parties' first, then 0, then i;
+        // slot k + 1: the digits of v.
+        auto poly_of = [k](int s, int i) { return s < k - 1 ? (s + 1 < i ? s + 1 : s + 2) : (s == k - 1 ? 0 : i); };
+        auto next_step = [&](int s) {  // e = 0: X^0 - 1 = 0, every digit is 0, the product adds nothing
+            while (s < limit && abar[s] == 0) ++s;
+            return s;
+        };
+        bool started = false;  // slot 0's products of this step are under way
+        int next = 0;
 #pragma unroll 1
-                for (int s = 0; s <= k + 1; ++s) {
-                    const int jj = s < k - 1 ? (s + 1 < i ? s + 1 : s + 2) : (s == k - 1 ? 0 : i);
-                    if (s <= k) {
-                        const uint32_t *ap = acc + jj * N;
-                        uint32_t w[8];
+        for (int step = next_step(0); step < limit; step = next) {
+            const int i = step / n + 1;
+            const uint32_t e = abar[step];
+            next = next_step(step + 1);
+            const uint4 *bk = bk_all + (size_t)step * 9 * POLY + pr * (POLY / 2);
+            uint32_t V[16];
 #pragma unroll
-                        for (int i8 = 0; i8 < 8; ++i8) {
-                            const uint32_t r = m0 + 16 * (i8 & 1) + 256 * (i8 >> 1) + e;
-                            const uint32_t a = ap[acc_pos(r & (N - 1))];
-                            const uint32_t neg = (uint32_t)((int32_t)(r << 21) >> 31);  // bit 10 of r: -1
-                            w[i8] = (a ^ neg) - neg - ap[(sw0 ^ (16 * (i8 & 1))) + 256 * (i8 >> 1)] + gad.offset;
-                        }
-                        store_digits(unit, w);
+            for (int c = 0; c < 16; ++c) V[c] = 0;
+            if (!started) {
+                cut_digits(poly_of(0, i), e);
+                start_products();
+            }
+            // The next step's first slot can start in this step's last one if its polynomial is final by then:
+            // another party's, so not one of this step's 0 and i.
+            started = k > 1 && next < limit && next / n + 1 == i;
+#pragma unroll 1
+            for (int s = 0; s <= k + 1; ++s) {
+                const int jj = poly_of(s, i);
+                if (!st_mbar_try(mbar, phase & 1)) products_wait(mbar, phase & 1, &ctl->abort, S.wait_ns, K.status);
+                ++phase;
+                __syncwarp();
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                uint32_t x[3][16];
+                load_factor(x[0], tmem_mine, q);
+                load_factor(x[1], tmem_mine + 16, q);
+                load_factor(x[2], tmem_mine + 32, q);
+                // the next slot's products run under this one's butterflies
+                if (s < k || (s == k + 1 && started)) {
+                    cut_digits(s < k ? poly_of(s + 1, i) : poly_of(0, i), s < k ? e : abar[next]);
+                    start_products();
+                }
+                // R1 = <x, key1>, R2 = <x, key2> in place of x[0], x[1]: (d, A_jj), or (f0, f1) of v's digits
+                const uint4 *k1 = bk + (s <= k ? 0 : 3 * POLY);
+                const uint4 *k2 = s <= k ? keyA + (size_t)jj * 3 * POLY + pr * (POLY / 2) : bk + 6 * POLY;
+                uint4 key[6];  // the first group is on its way during the butterflies
+                load_keys(key, k1, k2, half_odd, eighth);
+                half_stage<3, 3>(x, heap, q);
+                half_stage<3, 2>(x, heap, q);
+                half_stage<3, 1>(x, heap, q);
+                half_stage<3, 0>(x, heap, q);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+#pragma unroll
+                    for (int e4 = 0; e4 < 4; ++e4) {
+                        const int c = 4 * v + e4;
+                        const uint32_t x0 = x[0][c], x1 = x[1][c], x2 = x[2][c];
+                        x[0][c] = mac3_redc(x0, x1, x2, word_of(key[0], e4), word_of(key[1], e4), word_of(key[2], e4), q);
+                        x[1][c] = mac3_redc(x0, x1, x2, word_of(key[3], e4), word_of(key[4], e4), word_of(key[5], e4), q);
                     }
-                    st_fence_proxy_async();
-                    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                    quad_sync(bar);
-                    if (warp == 0 && lane == 0) {
-                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                        issue_products(tmem, start_s, planes_s, ones_s, digits_s, mbar);
-                    }
-                    __syncwarp();
-                    if (!st_mbar_try(mbar, phase & 1)) products_wait(mbar, phase & 1, &ctl->abort, S.wait_ns, K.status);
-                    ++phase;
-                    __syncwarp();
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    uint32_t x[3][16];
-                    load_factor(x[0], tmem_mine, q);
-                    load_factor(x[1], tmem_mine + 16, q);
-                    load_factor(x[2], tmem_mine + 32, q);
-                    half_stage<3, 3>(x, heap, q);
-                    half_stage<3, 2>(x, heap, q);
-                    half_stage<3, 1>(x, heap, q);
-                    half_stage<3, 0>(x, heap, q);
-                    // R1 = <x, key1>, R2 = <x, key2> in place of x[0], x[1]: (d, A_jj), or (f0, f1) of v's digits
-                    const uint4 *k1 = bk + (s <= k ? 0 : 3 * POLY);
-                    const uint4 *k2 = s <= k ? keyA + (size_t)jj * 3 * POLY + pr * (POLY / 2) : bk + 6 * POLY;
+                    if (v < 3) load_keys(key, k1, k2, half_odd + v + 1, eighth);
+                }
+                // phase A: v += R2, R1 is c'_jj; phase B: c'_0 += R1, c'_i (kept in V) += R2
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    const uint32_t a = V[c] + x[1][c];
+                    V[c] = min(a, a - q.p4);
+                }
+                if (s == k - 1) {
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) park[32 * v] = make_uint4(x[0][4 * v], x[0][4 * v + 1], x[0][4 * v + 2], x[0][4 * v + 3]);
+                    continue;
+                }
+                if (s == k + 1) {
 #pragma unroll
                     for (int v = 0; v < 4; ++v) {
-                        const uint32_t low = half_odd + v, pos = low * 32 + (eighth ^ low);
-                        uint4 ka[3], kb[3];
-#pragma unroll
-                        for (int l = 0; l < 3; ++l) {
-                            ka[l] = __ldg(k1 + l * POLY + pos);
-                            kb[l] = __ldg(k2 + l * POLY + pos);
-                        }
+                        const uint4 o = park[32 * v];
 #pragma unroll
                         for (int e4 = 0; e4 < 4; ++e4) {
-                            const int c = 4 * v + e4;
-                            const uint32_t x0 = x[0][c], x1 = x[1][c], x2 = x[2][c];
-                            x[0][c] = mac3_redc(x0, x1, x2, word_of(ka[0], e4), word_of(ka[1], e4), word_of(ka[2], e4), q);
-                            x[1][c] = mac3_redc(x0, x1, x2, word_of(kb[0], e4), word_of(kb[1], e4), word_of(kb[2], e4), q);
-                        }
-                    }
-                    // phase A: v += R2, R1 is c'_jj; phase B: c'_0 += R1, c'_i (kept in V) += R2
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        const uint32_t a = V[c] + x[1][c];
-                        V[c] = min(a, a - q.p4);
-                    }
-                    if (s == k - 1) {
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) park[32 * v] = make_uint4(x[0][4 * v], x[0][4 * v + 1], x[0][4 * v + 2], x[0][4 * v + 3]);
-                        continue;
-                    }
-                    if (s == k + 1) {
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            const uint4 o = park[32 * v];
-#pragma unroll
-                            for (int e4 = 0; e4 < 4; ++e4) {
-                                const uint32_t a = word_of(o, e4) + x[0][4 * v + e4];
-                                x[0][4 * v + e4] = min(a, a - q.p4);
-                            }
-                        }
-                    }
-                    // Inverse transforms due: the others' c'; v; c'_0 and c'_i
-                    const int jobs = s == k + 1 ? 2 : 1;
-#pragma unroll 1
-                    for (int job = 0; job < jobs; ++job) {
-                        uint32_t y[16], z[8];
-                        if (s != k) {
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) {
-                                y[c] = x[0][c];
-                                x[0][c] = V[c];  // the second job's
-                            }
-                        }
-                        else if (s == k) {
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) {
-                                y[c] = V[c];
-                                V[c] = x[0][c];
-                            }
-                        }
-                        inverse_crt(y, z, heap_rev, rows, crosses + pr * 16, crosses, xb, ex, q, h, warp, lane, bar);
-                        if (s == k) {
-#pragma unroll
-                            for (int c = 0; c < 8; ++c) z[c] += gad.offset;
-                            store_digits(unit, z);
-                        } else {
-                            uint32_t *ap = acc + (s == k + 1 ? (job ? i : 0) : jj) * N;
-#pragma unroll
-                            for (int c = 0; c < 8; ++c) ap[(sw0 ^ (16 * (c & 1))) + 256 * (c >> 1)] += z[c];
+                            const uint32_t a = word_of(o, e4) + x[0][4 * v + e4];
+                            x[0][4 * v + e4] = min(a, a - q.p4);
                         }
                     }
                 }
-                quad_sync(bar);
+                // Inverse transforms due: the others' c'; v; c'_0 and c'_i
+                const int jobs = s == k + 1 ? 2 : 1;
+#pragma unroll 1
+                for (int job = 0; job < jobs; ++job) {
+                    uint32_t y[16], z[8];
+                    if (s != k) {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) {
+                            y[c] = x[0][c];
+                            x[0][c] = V[c];  // the second job's
+                        }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) {
+                            y[c] = V[c];
+                            V[c] = x[0][c];
+                        }
+                    }
+                    inverse_crt(y, z, heap_rev, rows, crosses + pr * 16, crosses, xb, ex, q, h, warp, lane, bar);
+                    if (s == k) {
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) z[c] += gad.offset;
+                        store_digits(unit, z);
+                        start_products();
+                    } else {
+                        uint32_t *ap = acc + (s == k + 1 ? (job ? i : 0) : jj) * N;
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) ap[(sw0 ^ (16 * (c & 1))) + 256 * (c >> 1)] += z[c];
+                    }
+                }
             }
+            quad_sync(bar);
         }
         if (acc_out) {
             uint32_t *dst = acc_out + (size_t)gate * (k + 1) * N;
