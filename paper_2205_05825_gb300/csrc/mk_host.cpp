@@ -160,6 +160,8 @@ void free_device(mk_ctx *c) {
     cudaFree(c->d_bk);
     cudaFree(c->d_keyA);
     cudaFree(c->d_ks);
+    cudaFree(c->d_ksp);
+    c->d_ksp = nullptr;
     cudaFree(c->d_status);
     c->d_status = nullptr;
     cudaFree(c->d_ext);
@@ -410,6 +412,16 @@ int ensure_device_keys(mk_ctx *c) {
     for (uint32_t i = 0; i < k; ++i)
         MK_CUDA(c, cudaMemcpy(c->d_ks + (size_t)i * c->ks_words(), c->party[i].ks.data(), c->ks_words() * 4,
                               cudaMemcpyHostToDevice));
+    if (const size_t bytes = keyswitch_planes_bytes(c->shape())) {
+        if (!c->d_ksp && cudaMalloc(&c->d_ksp, bytes) != cudaSuccess) {
+            c->d_ksp = nullptr;  // no room: the key switch runs its kernels on the plain rows
+            (void)cudaGetLastError();
+        }
+        if (c->d_ksp) {
+            MK_CUDA(c, cudaStreamSynchronize(cudaStreamLegacy));  // the rows have landed
+            MK_CUDA(c, build_keyswitch_planes(c->shape(), c->d_ks, c->d_ksp, c->stream));
+        }
+    }
     c->cluster_cap = (uint32_t)cluster_capacity(c->shape());
     (void)cudaGetLastError();  // a shape the device cannot host only leaves the capacity at 0
     c->dev_keys_valid = true;
@@ -977,6 +989,8 @@ int mk_sync(mk_ctx *c) {
             MK_CUDA(c, cudaMemset(c->d_status, 0, sizeof(st)));
             if (st & kStatusStaged)
                 return fail(c, MK_ETIMEOUT, "a bounded wait of the staged blind rotation for a key copy gave up");
+            if (st & kStatusKeyswitch)
+                return fail(c, MK_ETIMEOUT, "a bounded wait of the key switch for a key copy or product gave up");
             if (st & kStatusWarp)
                 return fail(c, MK_ETIMEOUT, "a matrix product of the blind rotation did not complete in time");
             if (st & kStatusCluster)

@@ -47,7 +47,7 @@ struct DeviceKeys {
     void *tc_ws;
     uint32_t tc_ws_gates;
     // The context's status word (device): a kernel whose bounded wait ran out
-    // sets its bit (kStatusStaged, kStatusNetlist, kStatusCluster, kStatusWarp); mk_sync reports it as
+    // sets its bit (kStatusStaged, kStatusNetlist, kStatusCluster, kStatusWarp, kStatusKeyswitch); mk_sync reports it as
     // MK_ETIMEOUT and clears it.
     uint32_t *status;
     // MK_FORM_NTT2: per-prime twiddles [2 directions][2 primes][N] uint2
@@ -56,13 +56,17 @@ struct DeviceKeys {
     // MK_FORM_NTT2 at N = 1024: the warp kernel's tables (kWarpTableBytes,
     // layout in mk_bootstrap_warp.cuh); nullptr otherwise.
     const void *tw_warp;
+    // The key-switching keys as operand blocks of the matrix-product key
+    // switch (mk_keyswitch_tc.cu); nullptr where it does not apply.
+    const void *ks_planes;
 };
 
 // Tables of the warp kernel: twiddles by factor and by stage, matrix operands.
 constexpr size_t kWarpTableBytes = 16 * (2 * 2 * 8 * 32 + 2 * 16 + 2 * 16 + 2 * 128 + 3 * 4 * 256 + 2 * 48);
 constexpr size_t kWarpSmemMax = 227 * 1024;
 
-constexpr uint32_t kStatusStaged = 1u, kStatusNetlist = 2u, kStatusCluster = 4u, kStatusWarp = 8u;
+constexpr uint32_t kStatusStaged = 1u, kStatusNetlist = 2u, kStatusCluster = 4u, kStatusWarp = 8u,
+                   kStatusKeyswitch = 16u;
 
 struct LaunchShape {
     uint32_t n, N, logN, k, d, bg_bit, ks_bit, t;
@@ -236,11 +240,18 @@ cudaError_t launch_negacyclic_tc(uint32_t N, uint32_t G, uint32_t nchunks, const
 cudaError_t launch_mma_peak(uint32_t blocks, uint32_t threads, uint32_t iters, float *sink, cudaStream_t st);
 
 // a9: per-party key switch of ext [count][k*N+1] into out rows desc[g].out
-// (or row g when desc == nullptr).  From kKeyswitchBatchMin gates on (and for
-// 2-bit digits) a CTA serves a group of gates from each key row it reads.
+// (or row g when desc == nullptr): the matrix-product kernel where the keys
+// have its operand blocks (2-bit digits, t = 8), else a SIMT kernel: for 2-bit
+// digits and at least kKeyswitchBatchMin gates one whose CTA serves a group of
+// gates from each key row it reads, otherwise one CTA per gate.
 constexpr uint32_t kKeyswitchBatchMin = 64;
 cudaError_t launch_keyswitch(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
                              const uint32_t *ext, uint32_t *out, uint32_t count, cudaStream_t st);
+bool keyswitch_tc_supported(const LaunchShape &S);
+size_t keyswitch_planes_bytes(const LaunchShape &S);  // 0 where it does not apply
+cudaError_t build_keyswitch_planes(const LaunchShape &S, const uint32_t *ks, void *planes, cudaStream_t st);
+cudaError_t launch_keyswitch_tc(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc, const uint32_t *ext,
+                                uint32_t *out, uint32_t count, cudaStream_t st);
 
 // Eq. 8: out = (0, 1/4) - in.
 cudaError_t launch_not(const LaunchShape &S, const uint32_t *in, uint32_t *out, size_t count,

@@ -60,7 +60,8 @@ __global__ void keyswitch_kernel(LaunchShape S, const uint32_t *__restrict__ ks,
     }
 }
 
-// Batched key switch for 2-bit digits (three rows per digit level): a CTA
+// Batched key switch for 2-bit digits (three rows per digit level) where the
+// matrix-product kernel does not apply: a CTA
 // owns KS_GB gates and KS_CX output columns, so every key-switch row it reads
 // from L2 serves all its gates.  Per party i and block of KS_JB coefficients
 // the gates' digit words (a_{i,j} rounded to ks_bit*t bits) are staged in
@@ -441,6 +442,9 @@ cudaError_t launch_modswitch(const LaunchShape &S, const GateDesc *desc, const u
 cudaError_t launch_keyswitch(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
                              const uint32_t *ext, uint32_t *out, uint32_t count, cudaStream_t st) {
     if (count == 0) return cudaSuccess;
+    // 20 to 190 times the SIMT kernels' rate at every count from 1 to 4096 (figures in mk_keyswitch_tc.cu); they keep
+    // the digit layouts it does not take, and a context whose device had no room for the operand blocks.
+    if (K.ks_planes) return launch_keyswitch_tc(S, K, desc, ext, out, count, st);
     if (S.ks_bit == 2 && count >= kKeyswitchBatchMin) {
         const dim3 grid((count + KS_GB - 1) / KS_GB, (S.n + 1 + KS_CX - 1) / KS_CX);
         keyswitch_batched_kernel<<<grid, KS_CX, 0, st>>>(S, K.ks, desc, ext, out, count);
