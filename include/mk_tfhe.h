@@ -114,12 +114,15 @@ int mk_ctx_get_form(const mk_ctx *ctx, int *form);
 int mk_ctx_set_batch(mk_ctx *ctx, uint32_t max_gates_per_launch);
 
 /* Latency (cluster) form of the NTT blind rotation: one thread-block cluster
- * of k+1 CTAs per gate, CTA j owning accumulator polynomial j, so one gate
- * runs two to four times faster than in the batched kernel (k = 2 to 7)
- * while the GPU has SMs to spare.  MK_CLUSTER_AUTO (default) uses it for launches of at most
- * max(1, floor(k/2)) waves of gates, a wave being the clusters the device
- * can hold at once (queried when the keys are laid out for the form); _ON
- * for every launch, _OFF never.  Only the NTT forms with k <= 7; results are
+ * per gate, the k+1 accumulator polynomials spread over its CTAs, so one gate
+ * runs two to four times faster than in the batched kernels while the GPU has
+ * SMs to spare.  MK_FORM_NTT2 at N = 1024 with bg_bit 8: one to three
+ * polynomials per CTA (k <= 8); MK_CLUSTER_AUTO (default) takes the form, and
+ * the polynomials per CTA, that the launch's number of gates makes fastest
+ * (waves of the gates the device can hold at once, queried when the keys are
+ * laid out, times a measured time per wave).  Other shapes of the NTT forms:
+ * one polynomial per CTA, k <= 7; AUTO uses it for launches of at most
+ * max(1, floor(k/2)) waves.  _ON for every launch, _OFF never.  Results are
  * bit-identical either way.  No paper counterpart: a scheduling choice. */
 enum { MK_CLUSTER_AUTO = 0, MK_CLUSTER_OFF = 1, MK_CLUSTER_ON = 2 };
 int mk_ctx_set_cluster(mk_ctx *ctx, int mode);
@@ -133,7 +136,8 @@ int mk_ctx_set_cluster(mk_ctx *ctx, int mode);
  * without its outputs; the next mk_sync reports MK_ETIMEOUT, and the context
  * stays usable.  kind MK_FAULT_SKIP_KEY_STEP: until the next call, the staged
  * kernel and the cluster latency kernel never copy the key entry of CMux step
- * `arg` (0-based), so the waits for it run out.  kind MK_FAULT_SKIP_DIGIT_TILE: in the next tcgen05
+ * `arg` (0-based), or, where the latency form computes on the tensor cores,
+ * never start that step's products, so the waits for it run out.  kind MK_FAULT_SKIP_DIGIT_TILE: in the next tcgen05
  * launch, the first CTA that reaches its digit tile `arg` does not load it
  * (one shot).  kind MK_FAULT_SKIP_WIRE_READY: until the next call, the
  * persistent operator launch never marks the output of its work item `arg`

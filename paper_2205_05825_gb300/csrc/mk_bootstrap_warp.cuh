@@ -500,6 +500,16 @@ __device__ __forceinline__ void load_keys(uint4 (&key)[6], const uint4 *k1, cons
     }
 }
 
+// The same units of one key.
+__device__ __forceinline__ void load_key(uint4 (&key)[3], const uint4 *k1, uint32_t low, uint32_t eighth) {
+    const uint32_t pos = low * 32 + (eighth ^ low);
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+        asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(key[l].x), "=r"(key[l].y), "=r"(key[l].z), "=r"(key[l].w)
+                     : "l"(k1 + l * 512 + pos));
+}
+
 __device__ __forceinline__ uint32_t word_of(const uint4 &a, int h) {
     return h == 0 ? a.x : (h == 1 ? a.y : (h == 2 ? a.z : a.w));
 }

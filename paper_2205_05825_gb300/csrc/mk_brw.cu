@@ -1,5 +1,6 @@
-// Warp-level blind rotation (mk_bootstrap_warp.cuh): instantiation and launch.
-#include "mk_bootstrap_warp.cuh"
+// Warp and team blind rotations (mk_bootstrap_warp.cuh, mk_bootstrap_team.cuh):
+// instantiation, launch, and which of them a launch gets.
+#include "mk_bootstrap_team.cuh"
 
 namespace mk {
 namespace {
@@ -36,5 +37,66 @@ cudaError_t launch_bootstrap_warp(const LaunchShape &S, const DeviceKeys &K, con
     const uint32_t grid = count < (uint32_t)sms ? count : (uint32_t)sms;
     kern<<<grid, 128 * g, smem, st>>>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count);
     return cudaGetLastError();
+}
+
+void team_capacities(const LaunchShape &S, uint32_t cap[3]) {
+    cap[0] = cap[1] = cap[2] = 0;
+    if (!warp_form_supported(S)) return;
+    cap[0] = br::team_capacity<1>(S.k, S.n);
+    cap[1] = br::team_capacity<2>(S.k, S.n);
+    cap[2] = br::team_capacity<3>(S.k, S.n);
+}
+
+namespace {
+// Clocks of an SM (in thousands) that a CMux step takes, measured on GB300:
+// a full wave of the team kernel with 1, 2 and 3 teams a CTA (the same for k =
+// 1 to 8, polynomials run side by side; one share buffer costs a second
+// cluster barrier), and a pass of the warp kernel with 1, 2 and 3 gates a CTA,
+// per transform slot (k + 2 slots a step).
+constexpr double kTeamStep[3] = {14.5, 16.8, 23.5}, kOneBuffer = 2.5, kWarpSlot[3] = {6.8, 9.8, 11.5};
+
+double team_cost(const LaunchShape &S, uint32_t count, int t) {
+    if (!S.team_cap[t]) return 1e30;
+    const double step = kTeamStep[t] + (br::team_layout(S.k, S.n, t + 1).share_buffers == 1 ? kOneBuffer : 0.0);
+    return step * ((count + S.team_cap[t] - 1) / S.team_cap[t]);
+}
+
+double warp_cost(const LaunchShape &S, uint32_t count, uint32_t sms) {
+    const uint32_t g = warp_gates(S.k, S.n, 0xFFFFFFFFu / 2, sms), pass = g * sms;
+    if (g == 0) return 1e30;
+    const uint32_t rest = count % pass;
+    return (S.k + 2) * ((count / pass) * kWarpSlot[g - 1] + (rest ? kWarpSlot[(rest - 1) / sms] : 0.0));
+}
+
+// The team kernel's teams a CTA for this launch, less one; -1: not its launch.
+int team_choice(const LaunchShape &S, uint32_t count) {
+    if (S.cluster_mode == MK_CLUSTER_OFF || !warp_form_supported(S)) return -1;
+    int best = 0;
+    for (int t = 1; t < 3; ++t)
+        if (team_cost(S, count, t) < team_cost(S, count, best)) best = t;
+    if (!S.team_cap[best]) return -1;
+    if (S.cluster_mode == MK_CLUSTER_ON) return best;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return -1;
+    return team_cost(S, count, best) < warp_cost(S, count, (uint32_t)sms) ? best : -1;
+}
+}  // namespace
+
+bool team_form_chosen(const LaunchShape &S, uint32_t count) { return team_choice(S, count) >= 0; }
+
+cudaError_t launch_bootstrap_team(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
+                                  const uint32_t *ct_a, const uint32_t *ct_b, const uint32_t *abar_in,
+                                  int64_t max_steps, uint32_t *ext, uint32_t *acc_out, uint32_t count,
+                                  cudaStream_t st) {
+    if (count == 0) return cudaSuccess;
+    if (K.tw_warp == nullptr || K.status == nullptr) return cudaErrorInvalidValue;
+    switch (team_choice(S, count)) {
+        case 0: return br::launch_team<1>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count, st);
+        case 1: return br::launch_team<2>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count, st);
+        case 2: return br::launch_team<3>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count, st);
+        default: return cudaErrorInvalidConfiguration;
+    }
 }
 }  // namespace mk

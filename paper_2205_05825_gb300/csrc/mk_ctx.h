@@ -338,6 +338,7 @@ struct mk_ctx {
     int circuit_exec = MK_EXEC_AUTO;      // operators: one launch pair per level, or one persistent launch
     int64_t debug_skip_item = -1;         // test hook of the persistent launch (mk_debug_fault)
     uint32_t sm_count = 0;
+    uint32_t team_cap[3] = {0, 0, 0};  // resident gates of the team kernel, by teams a CTA (team_capacities)
     uint32_t cluster_cap = 0;  // resident clusters of the latency form for the keys' form (0: none)
     cudaStream_t capture_stream = nullptr;  // non-default stream the graphs are captured on
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev[2];
@@ -362,8 +363,8 @@ struct mk_ctx {
         const uint32_t cmax = cluster_mode == MK_CLUSTER_ON    ? 0xFFFFFFFFu
                               : cluster_mode == MK_CLUSTER_OFF ? 0u
                                                                : waves * cluster_cap;
-        return LaunchShape{P.n, P.N, logN, P.k, P.d, P.bg_bit, P.ks_bit, P.t, variant, form, cmax, wait_ns,
-                           debug_skip_key_step};
+        return LaunchShape{P.n, P.N, logN, P.k, P.d, P.bg_bit, P.ks_bit, P.t, variant, form, cmax,
+                           cluster_mode, {team_cap[0], team_cap[1], team_cap[2]}, wait_ns, debug_skip_key_step};
     }
     DeviceKeys dkeys() const {
         // twiddles: [2][N] of 8-byte (NTT) or 16-byte (NTT2) entries; FFT: one [3][N/2] table

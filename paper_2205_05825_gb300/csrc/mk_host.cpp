@@ -423,6 +423,7 @@ int ensure_device_keys(mk_ctx *c) {
         }
     }
     c->cluster_cap = (uint32_t)cluster_capacity(c->shape());
+    team_capacities(c->shape(), c->team_cap);
     (void)cudaGetLastError();  // a shape the device cannot host only leaves the capacity at 0
     c->dev_keys_valid = true;
     return MK_OK;

@@ -75,6 +75,10 @@ struct LaunchShape {
     // Batches of at most this many gates run the cluster (latency) kernel of
     // the NTT forms: one CTA per accumulator polynomial (0: never).
     uint32_t cluster_max;
+    // Latency forms of the warp kernel's shapes: MK_CLUSTER_* and, per teams a
+    // CTA (1, 2, 3), the gates resident at once (team_capacities).
+    int cluster_mode;
+    uint32_t team_cap[3];
     // Bound on each wait of the staged kernel for a key copy, in ns of global
     // time, and a test hook: the key copies of this CMux step are never
     // issued, so the waits for them run out (-1: none).
@@ -153,6 +157,18 @@ cudaError_t launch_bootstrap_warp(const LaunchShape &S, const DeviceKeys &K, con
                                   const uint32_t *ct_a, const uint32_t *ct_b, const uint32_t *abar_in,
                                   int64_t max_steps, uint32_t *ext, uint32_t *acc_out, uint32_t count,
                                   cudaStream_t st);
+
+// The latency form on the same shapes (mk_bootstrap_team.cuh): a cluster a
+// gate, a team of four warps a polynomial.  cap[t - 1]: gates resident at once
+// with t teams a CTA (0: the shape does not fit).
+void team_capacities(const LaunchShape &S, uint32_t cap[3]);
+cudaError_t launch_bootstrap_team(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
+                                  const uint32_t *ct_a, const uint32_t *ct_b, const uint32_t *abar_in,
+                                  int64_t max_steps, uint32_t *ext, uint32_t *acc_out, uint32_t count,
+                                  cudaStream_t st);
+// Whether launch_bootstrap_team takes a launch of `count` gates (its mode, and
+// under MK_CLUSTER_AUTO whether it is the faster form).
+bool team_form_chosen(const LaunchShape &S, uint32_t count);
 
 // Cluster (latency) form of the NTT blind rotation, one translation unit per
 // (ring dimension, field): mk_brc.cu built with -DMK_LOGN -DMK_FIELD.  Same

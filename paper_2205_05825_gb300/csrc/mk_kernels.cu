@@ -386,6 +386,8 @@ BootstrapFn pick(const LaunchShape &S) {
 
 // The cluster (latency) launcher for this shape and batch, or nullptr.
 BootstrapFn pick_cluster(const LaunchShape &S, uint32_t count) {
+    if (warp_form_supported(S) && S.k <= 8 && (S.team_cap[0] | S.team_cap[1] | S.team_cap[2]))
+        return team_form_chosen(S, count) ? launch_bootstrap_team : nullptr;
     if (count > S.cluster_max || S.k + 1 > 8 || (S.form != MK_FORM_NTT && S.form != MK_FORM_NTT2)) return nullptr;
     if (S.logN == 8) return S.form == MK_FORM_NTT ? launch_cluster_logn8_f0 : launch_cluster_logn8_f1;
     if (S.logN == 10) return S.form == MK_FORM_NTT ? launch_cluster_logn10_f0 : launch_cluster_logn10_f1;
