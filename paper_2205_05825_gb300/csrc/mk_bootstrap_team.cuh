@@ -52,7 +52,7 @@ struct TeamLayout {
 
 __host__ __device__ inline TeamLayout team_layout(uint32_t k, uint32_t n, uint32_t teams) {
     TeamLayout L;
-    L.ctl = (size_t)kTabUnits * 16;
+    L.ctl = (size_t)(teams == 3 ? Operands<3>::units : kTabSmall) * 16;
     L.team = L.ctl + ((sizeof(WarpCtl) + 15) & ~size_t(15));
     L.acc = 0;
     L.digits = 4096;
@@ -85,10 +85,10 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
     uint4 *tab = reinterpret_cast<uint4 *>(smem);
     {
         const uint4 *src = static_cast<const uint4 *>(K.tw_warp);
-        for (int u = threadIdx.x; u < kTabUnits; u += 128 * T) tab[u] = src[u];
+        for (int u = threadIdx.x; u < Operands<T>::units; u += 128 * T) tab[u] = src[u];
     }
     WarpCtl *ctl = reinterpret_cast<WarpCtl *>(smem + L.ctl);
-    constexpr uint32_t columns = T == 1 ? 256 : 512;
+    constexpr uint32_t columns = Operands<T>::columns;
     if (threadIdx.x == 0) {
         for (int g = 0; g < kWarpMaxGates; ++g) st_mbar_init(st_smem_addr(&ctl->bar[g]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -112,6 +112,10 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const int wid = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
+    if (wid < 4) fill_operands<T>(ctl->tmem, static_cast<const uint4 *>(K.tw_warp), wid, threadIdx.x & 31);
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const int lane = threadIdx.x & 31, warp = wid & 3, slot = wid >> 2, t128 = threadIdx.x & 127;
     const int pr = warp >> 1, h = warp & 1, bar = 1 + slot;
     const int jj = cta * T + slot;  // this team's polynomial
@@ -124,8 +128,8 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
     const uint4 *heap = tab + warp * 256 + lane, *heap_rev = tab + (warp ^ 1) * 256 + 31 - lane;
     const uint4 *rows = tab + kTabHalves + pr * 16;
     const uint4 *crosses = tab + kTabHalves + kTabRows;
-    const uint32_t start_s = st_smem_addr(crosses + kTabCross), planes_s = start_s + 16 * kTabStart;
-    const uint32_t ones_s = planes_s + 16 * kTabPlanes, digits_s = st_smem_addr(digits);
+    const uint32_t ones_s = st_smem_addr(crosses + kTabCross), plane0_s = ones_s + 16 * kTabOnes;
+    const uint32_t digits_s = st_smem_addr(digits);
     const uint32_t mbar0 = st_smem_addr(&ctl->bar[0]), tmem0 = ctl->tmem, lanes = (uint32_t)(32 * warp) << 16;
     const PrimeK q = prime_of(pr);
     const Gadget gad = make_gadget(8);
@@ -146,7 +150,7 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
         quad_sync(bar);
         if (warp == 0 && lane == 0 && issue) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            issue_products(tmem0 + 144 * slot, start_s, planes_s, ones_s, digits_s, mbar0 + 8 * slot);
+            issue_products<T>(tmem0, tmem0 + 144 * slot, ones_s, plane0_s, digits_s, mbar0 + 8 * slot);
         }
         __syncwarp();
     };
@@ -179,11 +183,19 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
     cluster_arrive();  // every CTA of the cluster is running before remote stores
     cluster_wait();
     uint32_t parity = 0;
+    int i = 1, left = n;  // party of the step, steps left of it
+    uint32_t e_next = abar[0];
 #pragma unroll 1
     for (int step = 0; step < limit; ++step) {
-        const uint32_t e = abar[step];
+        const uint32_t e = e_next;
+        e_next = abar[step + 1];  // (the last one reads b's word)
+        if (left == 0) {
+            left = n;
+            ++i;
+        }
+        --left;
         if (e == 0) continue;  // the same word in every CTA: the whole cluster skips
-        const int i = step / n + 1, cta_i = i / T;
+        const int cta_i = i / T;
         // The team of this CTA that transforms v, if the CTA holds polynomial 0 or i
         const int vteam = cta == 0 ? 0 : (cta == cta_i ? i % T : -1);
         const bool last = jj == 0 || jj == i;

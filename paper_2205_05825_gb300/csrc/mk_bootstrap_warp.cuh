@@ -105,20 +105,38 @@ __device__ __forceinline__ PrimeK prime_of(int pr) {
 //     forward twiddle 64 b + b y + i (entry 0 unused);
 //   rows [2][16]: entries 2u, 2u + 1 of forward twiddles 32 .. 63 (stage six of row f);
 //   cross [2][16]: entries 2u, 2u + 1 of forward twiddles 0 .. 31 (0 unused);
-//   start [2]: unit 0 (8 K slots x 128 rows) of the A operand's constant K
-//     step: 3072, then the offset B of plane 0 as 64 b1 + b0, or of planes 1,
-//     2 as 0 (its unit 1 is whatever follows: it meets zeros);
-//   planes [3][4 K steps]: A operand blocks (128 rows x 16 K slots, fp16) of
-//     the planes of zeta_y^s, row 64 prime + y; K slot 8 a + i stands for
+//   ones: the B operand's constant K step (48 columns): 4096, 64, 1, zeros;
+//   planes [3][4 K steps][2 units][128 rows]: A operand (fp16, 8 K slots a
+//     unit): the planes of zeta_y^s, row 64 prime + y; K slot 8 a + i stands for
 //     s = 2 a + 16 (i / 2) + i % 2;
-//   ones: the B operand's constant K step (48 columns): 4096, 64, 1, zeros.
-// Operand blocks are K-major without swizzle: 8 rows x 16 bytes contiguous,
-// row groups 128 bytes apart, K units of A 2048 and of B 768 bytes apart.
-constexpr int kTabHalves = 2 * 2 * 8 * 32, kTabRows = 2 * 16, kTabCross = 2 * 16;
-constexpr int kTabStart = 2 * 128, kTabPlanes = 3 * 4 * 256, kTabOnes = 2 * 48;
-constexpr int kTabUnits = kTabHalves + kTabRows + kTabCross + kTabStart + kTabPlanes + kTabOnes;
+//   start [2][128 rows]: unit 0 of the A operand's constant K step (its unit 1
+//     is zero): 3072, then the offset B of plane 0 as 64 b1 + b0, or 0 for
+//     planes 1 and 2.
+// The first four blocks and, where TMEM has no room for it, plane 0 are copied
+// into shared memory; the rest of the A operand goes into TMEM (rows = lanes,
+// two K slots a column), where the tensor core reads it without competing for
+// shared memory: with all of it there a step's products took 15 x 5.6 KB of
+// shared-memory reads.  Operand blocks in shared memory are K-major without
+// swizzle: 8 rows x 16 bytes contiguous, row groups 128 bytes apart, K units
+// of A 2048 and of B 768 bytes apart.
+constexpr int kTabHalves = 2 * 2 * 8 * 32, kTabRows = 2 * 16, kTabCross = 2 * 16, kTabOnes = 2 * 48;
+constexpr int kTabPlane = 4 * 256, kTabStart = 2 * 128;
+constexpr int kTabSmall = kTabHalves + kTabRows + kTabCross + kTabOnes;
+constexpr int kTabUnits = kTabSmall + 3 * kTabPlane + kTabStart;
 static_assert(kTabUnits * 16 == kWarpTableBytes, "table block");
 constexpr uint32_t kAUnit = 2048, kBUnit = 768;  // K-unit strides in bytes
+
+// A CTA with D gates (or teams): 144 TMEM columns each, then the constant
+// steps (8 columns each) and the planes (32 each), plane 0 in shared memory if
+// D = 3.
+template <int D>
+struct Operands {
+    static constexpr int first = D == 3 ? 1 : 0;  // first plane in TMEM
+    static constexpr uint32_t start = 144 * D, planes = start + 16, used = planes + 32 * (3 - first);
+    static constexpr uint32_t columns = used <= 256 ? 256 : 512;
+    static constexpr int units = kTabSmall + first * kTabPlane;  // table units in shared memory
+    static_assert(used <= 512, "TMEM columns");
+};
 
 // ---------------------------------------------------------------- shared memory
 // A control block, then per gate: accumulators, digits (the B operand, 6 KB),
@@ -136,7 +154,7 @@ struct WarpLayout {
 
 __host__ __device__ inline WarpLayout warp_layout(uint32_t k, uint32_t n, uint32_t gates) {
     WarpLayout L;
-    L.ctl = (size_t)kTabUnits * 16;
+    L.ctl = (size_t)Operands<kWarpMaxGates>::units * 16;
     L.gate = L.ctl + ((sizeof(WarpCtl) + 15) & ~size_t(15));
     L.acc = 0;
     L.digits = L.acc + (size_t)4096 * (k + 1);
@@ -217,23 +235,56 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t saddr, uint32_t k_stri
            (1ull << 46);
 }
 
-// One thread: the three planes' products of a gate's digits (15 MMAs) into
-// its 144 TMEM columns, then a commit to its mbarrier.
-__device__ __forceinline__ void issue_products(uint32_t tmem, uint32_t start, uint32_t planes, uint32_t ones,
+__device__ __forceinline__ void tmem_st8(uint32_t addr, const uint4 &a, const uint4 &b) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"r"(addr), "r"(a.x),
+                 "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+
+// Warps 0-3 of a CTA: their rows of the A operand into TMEM.
+template <int D>
+__device__ __forceinline__ void fill_operands(uint32_t tmem, const uint4 *table, int warp, int lane) {
+    using O = Operands<D>;
+    const uint32_t at = tmem + ((uint32_t)(32 * warp) << 16);
+    const uint4 *row = table + kTabSmall + 32 * warp + lane;
+#pragma unroll
+    for (int st = 0; st < 2; ++st)
+        tmem_st8(at + O::start + 8 * st, __ldg(row + 3 * kTabPlane + 128 * st), make_uint4(0, 0, 0, 0));
+#pragma unroll
+    for (int b = 4 * O::first; b < 12; ++b)
+        tmem_st8(at + O::planes + 8 * (b - 4 * O::first), __ldg(row + 256 * b), __ldg(row + 256 * b + 128));
+    asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+}
+
+// One thread: the three planes' products of the digits at `digits` (15 MMAs)
+// into the 144 TMEM columns at d, then a commit to the mbarrier.  tmem: the
+// CTA's columns; ones, plane0: shared-memory addresses.
+template <int D>
+__device__ __forceinline__ void issue_products(uint32_t tmem, uint32_t d, uint32_t ones, uint32_t plane0,
                                                uint32_t digits, uint32_t bar) {
+    using O = Operands<D>;
     const uint64_t bone = operand_desc(ones, kBUnit), bdig = operand_desc(digits, kBUnit);
-    const uint64_t astart = operand_desc(start, kAUnit), aplane = operand_desc(planes, kAUnit);
+    const uint64_t aplane = operand_desc(plane0, kAUnit);
 #pragma unroll
     for (int pl = 0; pl < 3; ++pl) {
 #pragma unroll
         for (int ks = -1; ks < 4; ++ks) {
-            const uint64_t ad = ks < 0 ? astart + (pl ? kAUnit / 16 : 0) : aplane + (pl * 4 + ks) * (2 * kAUnit / 16);
             const uint64_t bd = ks < 0 ? bone : bdig + ks * (2 * kBUnit / 16);
-            asm volatile(
-                "{\n\t.reg .pred p;\n\t"
-                "setp.ne.b32 p, %4, 0;\n\t"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem + 48 * pl),
-                "l"(ad), "l"(bd), "r"(kWarpIdesc), "r"(ks < 0 ? 0u : 1u));
+            const uint32_t acc = ks < 0 ? 0u : 1u;
+            if (ks >= 0 && pl < O::first) {
+                asm volatile(
+                    "{\n\t.reg .pred p;\n\t"
+                    "setp.ne.b32 p, %4, 0;\n\t"
+                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d + 48 * pl),
+                    "l"(aplane + ks * (2 * kAUnit / 16)), "l"(bd), "r"(kWarpIdesc), "r"(acc));
+            } else {
+                const uint32_t at = tmem + (ks < 0 ? O::start + (pl ? 8 : 0) : O::planes + 32 * (pl - O::first) + 8 * ks);
+                asm volatile(
+                    "{\n\t.reg .pred p;\n\t"
+                    "setp.ne.b32 p, %4, 0;\n\t"
+                    "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d + 48 * pl),
+                    "r"(at), "l"(bd), "r"(kWarpIdesc), "r"(acc));
+            }
         }
     }
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
@@ -527,10 +578,10 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
     uint4 *tab = reinterpret_cast<uint4 *>(smem);
     {
         const uint4 *src = static_cast<const uint4 *>(K.tw_warp);
-        for (int u = threadIdx.x; u < kTabUnits; u += blockDim.x) tab[u] = src[u];
+        for (int u = threadIdx.x; u < Operands<kWarpMaxGates>::units; u += blockDim.x) tab[u] = src[u];
     }
     WarpCtl *ctl = reinterpret_cast<WarpCtl *>(smem + L.ctl);
-    const uint32_t columns = G == 1 ? 256 : 512;
+    constexpr uint32_t columns = Operands<kWarpMaxGates>::columns;
     if (threadIdx.x == 0) {
         for (int g = 0; g < kWarpMaxGates; ++g) st_mbar_init(st_smem_addr(&ctl->bar[g]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -548,6 +599,10 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     // the warp's index by a shuffle: uniform to the compiler, so constants and bases need no vector registers
     const int wid = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
+    if (wid < 4) fill_operands<kWarpMaxGates>(ctl->tmem, static_cast<const uint4 *>(K.tw_warp), wid, threadIdx.x & 31);
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const int lane = threadIdx.x & 31, warp = wid & 3, slot = wid >> 2, t128 = threadIdx.x & 127;
     const int pr = warp >> 1, h = warp & 1, bar = 1 + slot;
     unsigned char *gm = smem + L.gate + L.gate_bytes * slot;
@@ -559,8 +614,8 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
     const uint4 *heap = tab + warp * 256 + lane, *heap_rev = tab + (warp ^ 1) * 256 + 31 - lane;
     const uint4 *rows = tab + kTabHalves + pr * 16;
     const uint4 *crosses = tab + kTabHalves + kTabRows;
-    const uint32_t start_s = st_smem_addr(crosses + kTabCross), planes_s = start_s + 16 * kTabStart;
-    const uint32_t ones_s = planes_s + 16 * kTabPlanes, digits_s = st_smem_addr(digits);
+    const uint32_t ones_s = st_smem_addr(crosses + kTabCross), plane0_s = ones_s + 16 * kTabOnes;
+    const uint32_t digits_s = st_smem_addr(digits);
     const uint32_t mbar = st_smem_addr(&ctl->bar[slot]);
     const uint32_t tmem = ctl->tmem + 144 * slot, tmem_mine = tmem + ((uint32_t)(32 * warp) << 16);
     const PrimeK q = prime_of(pr);
@@ -614,7 +669,7 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
             quad_sync(bar);
             if (warp == 0 && lane == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                issue_products(tmem, start_s, planes_s, ones_s, digits_s, mbar);
+                issue_products<kWarpMaxGates>(ctl->tmem, tmem, ones_s, plane0_s, digits_s, mbar);
             }
             __syncwarp();
         };

@@ -212,9 +212,9 @@ void warp_tables(const HostNtt32 &t1, const HostNtt32 &t2, unsigned char *out) {
     uint32_t *halves = reinterpret_cast<uint32_t *>(out);
     uint32_t *rows = halves + 4 * (2 * 2 * 8 * 32);
     uint32_t *cross = rows + 4 * (2 * 16);
-    uint16_t *start = reinterpret_cast<uint16_t *>(cross + 4 * (2 * 16));
-    uint16_t *planes = start + 8 * (2 * 128);
-    uint16_t *ones = planes + 8 * (3 * 4 * 256);
+    uint16_t *ones = reinterpret_cast<uint16_t *>(cross + 4 * (2 * 16));
+    uint16_t *planes = ones + 8 * (2 * 48);
+    uint16_t *start = planes + 8 * (3 * 4 * 256);
     // offsets B of the first plane (prime_of in mk_bootstrap_warp.cuh) as 64 b1 + b0
     const int b1[2] = {-256, -71}, b0[2] = {4, -7};
     for (uint32_t pr = 0; pr < 2; ++pr) {
