@@ -131,7 +131,7 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
     const uint32_t ones_s = st_smem_addr(crosses + kTabCross), plane0_s = ones_s + 16 * kTabOnes;
     const uint32_t digits_s = st_smem_addr(digits);
     const uint32_t mbar0 = st_smem_addr(&ctl->bar[0]), tmem0 = ctl->tmem, lanes = (uint32_t)(32 * warp) << 16;
-    const PrimeK q = prime_of(pr);
+    const PrimeK q = prime_of(pr, S.d - 3);
     const Gadget gad = make_gadget(8);
     const uint4 *bk_all = static_cast<const uint4 *>(K.bk) + pr * (POLY / 2);
     const uint4 *key_a = static_cast<const uint4 *>(K.keyA) + (size_t)jj * 3 * POLY + pr * (POLY / 2);
