@@ -484,7 +484,8 @@ int mk_measure_butterfly_rate(int device, void *stream, int form, uint32_t iters
  * MK_EINVAL.  MK_ETIMEOUT if a bounded wait of the tcgen05 kernel gave up.
  * The call allocates a bf16 copy of the digits, runs on `stream` and
  * synchronises it.  The same engine numbers select the tensor form's engine
- * as its variant (mk_ctx_set_variant; mk_autotune times both).
+ * as its variant (mk_ctx_set_variant; mk_autotune times both); every other
+ * variant number, the default among them, runs engine 1.
  * No paper counterpart: the negacyclic product of Sec. 3.1-3.2 (the hybrid
  * product's inner step) isolated for testing the tensor form. */
 int mk_tc_negacyclic(int device, void *stream, uint32_t N, uint32_t G, uint32_t nchunks, const uint32_t *keys,

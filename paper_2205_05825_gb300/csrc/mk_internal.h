@@ -233,12 +233,14 @@ struct TcArgs {
     const uint16_t *dig;
     size_t dig_zstride;
     int nchunks;
+    int split;       // tcgen05 engine, set by its launcher: one item per chunk, added atomically into dst
     int dig_chunks;  // digit polynomials in the whole dig array (for the tcgen05 engine's tensor map)
     uint64_t wait_ns;  // bound on each mbarrier wait of the tcgen05 engine (global time)
 };
 // The tcgen05 engine of those products (mk_tensor_tc05.cu): G a multiple of
 // 128; one persistent CTA per SM over (coefficient tile, gate tile, output)
-// items of 128 x 128.  tc05_error reads (and optionally clears) the timeout record of its
+// items of 128 x 128, or, where three times as many still fit the SMs in one
+// wave and dst is accumulated into, of one key polynomial each.  tc05_error reads (and optionally clears) the timeout record of its
 // bounded waits (0: none).
 cudaError_t launch_products_tc05(const TcArgs &A, uint32_t N, uint32_t G, int outputs, cudaStream_t st);
 cudaError_t tc05_error(unsigned int *code, bool clear);

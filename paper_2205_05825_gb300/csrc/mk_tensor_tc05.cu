@@ -252,6 +252,8 @@ __device__ __forceinline__ T5Item item_of(const TcArgs &A, uint32_t G, int it) {
     constexpr int N = 1 << LOGN, MT = N / T5_M;
     const int GT = (int)(G / T5_NG);
     T5Item r;
+    const int chunk = A.split ? it % A.nchunks : 0;
+    if (A.split) it /= A.nchunks;
     r.m0 = (it % MT) * T5_M;
     const int rest = it / MT;
     r.g0 = (uint32_t)(rest % GT) * T5_NG;
@@ -260,6 +262,8 @@ __device__ __forceinline__ T5Item item_of(const TcArgs &A, uint32_t G, int it) {
     r.zi = z >> 1;
     r.chunk0 = (int)(r.zi * (A.dig_zstride / ((size_t)G * N)));
     r.key = r.type ? A.key[1] + r.zi * A.key_zstride[1] : A.key[0] + r.zi * A.key_zstride[0];
+    r.chunk0 += chunk;
+    r.key += (size_t)chunk * N;
     return r;
 }
 
@@ -289,7 +293,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1)
     volatile uint32_t *abort = reinterpret_cast<volatile uint32_t *>(smem + L::off_abort);
     const uint64_t wait_ns = A.wait_ns;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nch = A.nchunks, PI = 2 * nch;  // passes per item
+    const int nch = A.split ? 1 : A.nchunks, PI = 2 * nch;  // key polynomials and passes per item
     const int my_items = (items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
     const int PT = my_items * PI;             // passes of this CTA
     unsigned char *abuf = smem + L::off_a;
@@ -444,6 +448,11 @@ __global__ void __launch_bounds__(T5_THREADS, 1)
                     const T5Item I = item_of<LOGN>(A, G, (int)blockIdx.x + (pp / PI) * (int)gridDim.x);
                     int32_t *dst = (I.type ? A.dst[1] : A.dst[0]) + I.zi * A.dst_zstride + (I.m0 + 127 - tid) +
                                    (size_t)I.g0 * A.dst_stride;
+                    if (A.split) {
+#pragma unroll 8
+                        for (int g = 0; g < T5_NG; ++g)
+                            atomicAdd(reinterpret_cast<uint32_t *>(dst) + (size_t)g * A.dst_stride, sacc[g * T5_M + tid]);
+                    } else
 #pragma unroll 1
                     for (int g = 0; g < T5_NG; g += 16) {
                         uint32_t old[16];
@@ -518,9 +527,14 @@ static cudaError_t launch_tc05(const TcArgs &A, uint32_t G, int outputs, cudaStr
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     // one CTA per SM (its shared memory and TMEM take the SM), each looping over items
-    const int items = (N / T5_M) * (int)(G / T5_NG) * outputs;
+    // A launch that leaves two thirds of the SMs idle gives each key polynomial its own item: the second product
+    // of a step at 384 gates is 48 items of 60 us, or 144 of a third (integer sums: the order does not matter).
+    int items = (N / T5_M) * (int)(G / T5_NG) * outputs;
+    TcArgs B = A;
+    B.split = A.accumulate && A.nchunks > 1 && items * A.nchunks <= sms;
+    if (B.split) items *= A.nchunks;
     const int grid = items < sms ? items : sms;
-    tc05_products_kernel<LOGN><<<grid, T5_THREADS, T5Smem<LOGN>::bytes, st>>>(A, G, items, map);
+    tc05_products_kernel<LOGN><<<grid, T5_THREADS, T5Smem<LOGN>::bytes, st>>>(B, G, items, map);
     return cudaGetLastError();
 }
 
