@@ -120,7 +120,9 @@ int mk_ctx_set_batch(mk_ctx *ctx, uint32_t max_gates_per_launch);
  * polynomials per CTA (k <= 8); MK_CLUSTER_AUTO (default) takes the form, and
  * the polynomials per CTA, that the launch's number of gates makes fastest
  * (waves of the gates the device can hold at once, queried when the keys are
- * laid out, times a measured time per wave).  Other shapes of the NTT forms:
+ * laid out, times a measured time per wave).  Under MK_FORM_NTT2 at N = 256
+ * with bg_bit 8 AUTO never takes it (variant 2 is faster).  Other shapes of the
+ * NTT forms:
  * one polynomial per CTA, k <= 7; AUTO uses it for launches of at most
  * max(1, floor(k/2)) waves.  _ON for every launch, _OFF never.  Results are
  * bit-identical either way.  No paper counterpart: a scheduling choice. */
@@ -200,8 +202,9 @@ int mk_ctx_get_circuit_style(const mk_ctx *ctx, int *style);
 /* Blind-rotation kernel variants (same results, different register/occupancy
  * trade-offs): 0..MK_NUM_VARIANTS-1.  0-5: one CTA per gate, with different
  * digit polynomials per forward pass, register caps, twiddle placement and
- * elements per thread (under MK_FORM_NTT2 at N = 1024 with bg_bit 8, 2 is the
- * warp kernel: tcgen05 products for the first transform stages); 6: several gates per CTA sharing each CMux step's
+ * elements per thread (under MK_FORM_NTT2 with bg_bit 8, 2 is the warp
+ * kernel at N = 1024, tcgen05 products for the first transform stages, and a
+ * warp per polynomial and prime at N = 256); 6: several gates per CTA sharing each CMux step's
  * bootstrapping-key entry, bulk-copied once into shared memory; 7, 8
  * (MK_FORM_NTT2): the two primes' transforms on separate warps, recombined
  * by CRT through shared memory (MK_FORM_NTT runs variant 2's kernel for 7

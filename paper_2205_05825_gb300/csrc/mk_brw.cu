@@ -1,5 +1,6 @@
 // Warp and team blind rotations (mk_bootstrap_warp.cuh, mk_bootstrap_team.cuh):
 // instantiation, launch, and which of them a launch gets.
+#include "mk_bootstrap_small.cuh"
 #include "mk_bootstrap_team.cuh"
 
 namespace mk {
@@ -98,5 +99,32 @@ cudaError_t launch_bootstrap_team(const LaunchShape &S, const DeviceKeys &K, con
         case 2: return br::launch_team<3>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count, st);
         default: return cudaErrorInvalidConfiguration;
     }
+}
+
+bool small_form_supported(const LaunchShape &S) {
+    return S.form == MK_FORM_NTT2 && S.logN == 8 && S.d == 3 && S.bg_bit == 8 && S.k <= 8 &&
+           br::small_layout(S.k, S.n).total <= kWarpSmemMax;
+}
+
+cudaError_t launch_bootstrap_small(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
+                                   const uint32_t *ct_a, const uint32_t *ct_b, const uint32_t *abar_in,
+                                   int64_t max_steps, uint32_t *ext, uint32_t *acc_out, uint32_t count,
+                                   cudaStream_t st) {
+    if (count == 0) return cudaSuccess;
+    if (!small_form_supported(S) || K.tw_split == nullptr) return cudaErrorInvalidValue;
+    const size_t smem = br::small_layout(S.k, S.n).total;
+    auto run = [&](auto kern) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<count, 64 * (S.k + 1), smem, st>>>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out);
+        return cudaGetLastError();
+    };
+    if (S.k > 3) return run(br::bootstrap_small_kernel<8, 1>);
+    // one gate an SM: all the registers; more: three CTAs an SM (600 gates at k = 2 1.38 ms, with two 1.45)
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    return count <= (uint32_t)sms ? run(br::bootstrap_small_kernel<3, 1>) : run(br::bootstrap_small_kernel<3, 3>);
 }
 }  // namespace mk

@@ -170,6 +170,14 @@ cudaError_t launch_bootstrap_team(const LaunchShape &S, const DeviceKeys &K, con
 // under MK_CLUSTER_AUTO whether it is the faster form).
 bool team_form_chosen(const LaunchShape &S, uint32_t count);
 
+// The two-prime form at N = 256, d = 3, bg_bit = 8 (mk_bootstrap_small.cuh):
+// one CTA a gate, one warp per polynomial and prime.
+bool small_form_supported(const LaunchShape &S);
+cudaError_t launch_bootstrap_small(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
+                                   const uint32_t *ct_a, const uint32_t *ct_b, const uint32_t *abar_in,
+                                   int64_t max_steps, uint32_t *ext, uint32_t *acc_out, uint32_t count,
+                                   cudaStream_t st);
+
 // Cluster (latency) form of the NTT blind rotation, one translation unit per
 // (ring dimension, field): mk_brc.cu built with -DMK_LOGN -DMK_FIELD.  Same
 // arguments as the launchers above; needs k + 1 <= 8.  cluster_capacity_*:

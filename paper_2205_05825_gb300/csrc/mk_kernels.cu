@@ -379,6 +379,8 @@ BootstrapFn pick(const LaunchShape &S) {
     // measured count it beats variant 2's own kernel (4096 gates, k = 2: 224 against 347 ms; one gate per SM:
     // 15 against 31 ms), which keeps the other shapes.
     if (S.variant == 2 && warp_form_supported(S)) return launch_bootstrap_warp;
+    // At N = 256 the small kernel does, at every measured count (figures in mk_bootstrap_small.cuh).
+    if (S.variant == 2 && small_form_supported(S)) return launch_bootstrap_small;
     if (S.logN == 8) return t8[S.form][S.variant];
     if (S.logN == 10) return t10[S.form][S.variant];
     return nullptr;
@@ -388,6 +390,9 @@ BootstrapFn pick(const LaunchShape &S) {
 BootstrapFn pick_cluster(const LaunchShape &S, uint32_t count) {
     if (warp_form_supported(S) && S.k <= 8 && (S.team_cap[0] | S.team_cap[1] | S.team_cap[2]))
         return team_form_chosen(S, count) ? launch_bootstrap_team : nullptr;
+    // At N = 256 the small kernel is faster than the cluster at every count.
+    if (S.cluster_mode == MK_CLUSTER_AUTO && small_form_supported(S))
+        return S.variant == 2 || count <= S.cluster_max ? launch_bootstrap_small : nullptr;
     if (count > S.cluster_max || S.k + 1 > 8 || (S.form != MK_FORM_NTT && S.form != MK_FORM_NTT2)) return nullptr;
     if (S.logN == 8) return S.form == MK_FORM_NTT ? launch_cluster_logn8_f0 : launch_cluster_logn8_f1;
     if (S.logN == 10) return S.form == MK_FORM_NTT ? launch_cluster_logn10_f0 : launch_cluster_logn10_f1;
