@@ -66,6 +66,16 @@ __host__ __device__ inline TeamLayout team_layout(uint32_t k, uint32_t n, uint32
     return L;
 }
 
+// One lane of the warp (the compiler keeps the uniform registers that the
+// matrix instructions take their operands from in such a branch: the issue of
+// a step's products is on the critical path here, one gate 6.75 -> 6.57 ms; the
+// warp kernel, where it is not, measured slower with it).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+    return r != 0;
+}
+
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 
@@ -148,7 +158,7 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
         st_fence_proxy_async();
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
         quad_sync(bar);
-        if (warp == 0 && lane == 0 && issue) {
+        if (warp == 0 && issue && elect_one()) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             issue_products<T>(tmem0, tmem0 + 144 * slot, ones_s, plane0_s, digits_s, mbar0 + 8 * slot);
         }
