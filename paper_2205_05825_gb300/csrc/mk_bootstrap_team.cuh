@@ -22,11 +22,12 @@
 // T teams a CTA, ceil((k + 1) / T) CTAs a cluster.  T = 1 has the shortest
 // step (a team has the SM's four schedulers to itself); T = 2 and 3 put more
 // gates on the chip at once.  Measured (GB300, blind rotation of one wave):
-// k = 2: 1 gate 6.8 ms (the cluster kernel it replaces 11.5, the warp kernel
-// 16.5), 37 gates 8.1, 76 gates (T = 2) 9.0, 152 gates (T = 3) 12.5 against 15.0;
-// k = 4: 1 gate 13.8 (23.7), 40 gates 18.2; k = 8: 1 gate 42 ms against 152.
-// A step is a chain of dependent phases (products, butterflies, two inverse
-// transforms, a cluster barrier): 12.6 k clocks at T = 1.
+// k = 2: 1 gate 6.4 ms (the cluster kernel it replaces 11.5, the warp kernel
+// 15.7), 37 gates 7.7, 76 gates (T = 2) 8.4, 152 gates (T = 3) 10.7 against 14.3;
+// k = 4: 1 gate 13.3 (23.7), 5 gates 13.5; k = 8: 1 gate 36 ms against 150.
+// A step is a chain of dependent phases: at T = 1 about 11.8 k clocks, of them
+// digits 0.6, two products 0.8 each, two sets of butterflies and key products
+// 2.3 and 1.9, the cluster barrier 1.0, two inverse transforms 1.4 each.
 // Waits for products are bounded (products_wait); a CTA whose wait ran out
 // keeps passing the cluster barriers, so it strands no other (its results are
 // garbage and mk_sync reports MK_ETIMEOUT).
@@ -171,9 +172,16 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
     };
     auto load_products = [&](uint32_t(&x)[3][16], int s) {
         const uint32_t tmem = tmem0 + 144 * s + lanes;
-        load_factor(x[0], tmem, q);
-        load_factor(x[1], tmem + 16, q);
-        load_factor(x[2], tmem + 32, q);
+        PlaneSums f[2];  // a digit's sums are on their way while the one before is combined
+        fetch_sums(f[0], tmem);
+        sums_fetched();
+        fetch_sums(f[1], tmem + 16);
+        combine_planes(x[0], f[0], q);
+        sums_fetched();
+        fetch_sums(f[0], tmem + 32);
+        combine_planes(x[1], f[1], q);
+        sums_fetched();
+        combine_planes(x[2], f[0], q);
     };
     auto butterflies = [&](uint32_t(&x)[3][16]) {
         half_stage<3, 3>(x, heap, q);
@@ -267,15 +275,17 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
             for (int c = 0; c < 8; ++c) acc[(sw0 ^ (16 * (c & 1))) + 256 * (c >> 1)] += z[c];
             quad_sync(bar);
         }
+        const uint4 *kf = bk + (jj == 0 ? 3 : 6) * POLY;
+        constexpr int FAHEAD = T == 1 ? 4 : 1;
+        uint4 key[FAHEAD][3];
+        if (last) {
+#pragma unroll
+            for (int v = 0; v < FAHEAD; ++v) load_key(key[v], kf, half_odd + v, eighth);
+        }
         __syncwarp();
         cluster_wait();  // every share of v has arrived
         if (last) {
             // 3. w = g^-1(v), c'_0 += <w, f0>, c'_i += <w, f1>
-            const uint4 *kf = bk + (jj == 0 ? 3 : 6) * POLY;
-            constexpr int AHEAD = T == 1 ? 4 : 1;
-            uint4 key[AHEAD][3];
-#pragma unroll
-            for (int v = 0; v < AHEAD; ++v) load_key(key[v], kf, half_odd + v, eighth);
             if (slot == vteam) {
                 uint32_t y[16];
                 const uint4 *src = shares + (size_t)parity * 512 * (k + 1) + t128;
@@ -314,12 +324,12 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
 #pragma unroll
                 for (int e4 = 0; e4 < 4; ++e4) {
                     const int c = 4 * v + e4;
-                    const uint4(&kv)[3] = key[v % AHEAD];
+                    const uint4(&kv)[3] = key[v % FAHEAD];
                     const uint32_t a = C[c] + mac3_redc(x[0][c], x[1][c], x[2][c], word_of(kv[0], e4), word_of(kv[1], e4),
                                                         word_of(kv[2], e4), q);
                     C[c] = min(a, a - q.p4);
                 }
-                if (v + AHEAD < 4) load_key(key[v % AHEAD], kf, half_odd + v + AHEAD, eighth);
+                if (v + FAHEAD < 4) load_key(key[v % FAHEAD], kf, half_odd + v + FAHEAD, eighth);
             }
             inverse_crt(C, z, heap_rev, rows, crosses + pr * 16, crosses, xb, ex, q, h, warp, lane, bar);
 #pragma unroll

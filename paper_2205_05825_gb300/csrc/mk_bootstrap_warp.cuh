@@ -43,10 +43,10 @@
 // step of a gate: on this chip it competes with the integer multiplies for
 // the register file, and its fragments need a transposition.)
 //
-// Measured (GB300, whole blind rotation): 4096 gates at k = 2 347 -> 224 ms,
-// 1001 at k = 4 308 -> 192 ms, 96 at k = 8 333 -> 146 ms, 152 at k = 2 (one gate
-// per SM) 31 -> 15.0 ms.  Per CMux step and gate 23.7 -> 15.4 k clocks of an SM;
-// the multiply pipe's own share is 10 k.
+// Measured (GB300, whole blind rotation): 4096 gates at k = 2 347 -> 211 ms,
+// 1001 at k = 4 308 -> 182 ms, 96 at k = 8 333 -> 139 ms, 152 at k = 2 (one gate
+// per SM) 31 -> 14.3 ms.  Per CMux step and gate 23.7 -> 14.5 k clocks of an SM;
+// the multiply pipe is 81 % busy (ncu, three gates an SM).
 //
 // A CTA holds G gates (4 G warps) and the tables once; the grid is at most one
 // CTA per SM and walks the gates with stride G * gridDim.
@@ -319,24 +319,35 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&r)[16]) {
         : "r"(addr));
 }
 
-// Elements of this thread's factor of one digit polynomial, below 3.6 p, from
-// its planes' sums at columns tmem, tmem + 48, tmem + 96.
-__device__ __forceinline__ void load_factor(uint32_t (&x)[16], uint32_t tmem, const PrimeK &q) {
+// Sums of the three planes for this thread's factor of one digit polynomial
+// (columns tmem, tmem + 48, tmem + 96), and the factor's elements from them,
+// below 3.6 p.
+struct PlaneSums {
     float f0[16], f1[16], f2[16];
-    tmem_ld16(tmem, f0);
-    tmem_ld16(tmem + 48, f1);
-    tmem_ld16(tmem + 96, f2);
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+};
+__device__ __forceinline__ void fetch_sums(PlaneSums &f, uint32_t tmem) {
+    tmem_ld16(tmem, f.f0);
+    tmem_ld16(tmem + 48, f.f1);
+    tmem_ld16(tmem + 96, f.f2);
+}
+__device__ __forceinline__ void sums_fetched() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void combine_planes(uint32_t (&x)[16], const PlaneSums &f, const PrimeK &q) {
 #pragma unroll
     for (int e = 0; e < 16; e += 2) {
         float g0, g1;
-        fma_pair(g0, g1, f1[e], f1[e + 1], q.c1, q.kf, q.kf);
-        fma_pair(g0, g1, f2[e], f2[e + 1], q.c2, g0, g1);
-        x[e] = __float_as_uint(f0[e]) + (__float_as_uint(f1[e]) << 9) + (__float_as_uint(f2[e]) << 18) -
+        fma_pair(g0, g1, f.f1[e], f.f1[e + 1], q.c1, q.kf, q.kf);
+        fma_pair(g0, g1, f.f2[e], f.f2[e + 1], q.c2, g0, g1);
+        x[e] = __float_as_uint(f.f0[e]) + (__float_as_uint(f.f1[e]) << 9) + (__float_as_uint(f.f2[e]) << 18) -
                __float_as_uint(g0) * q.p;
-        x[e + 1] = __float_as_uint(f0[e + 1]) + (__float_as_uint(f1[e + 1]) << 9) + (__float_as_uint(f2[e + 1]) << 18) -
-                   __float_as_uint(g1) * q.p;
+        x[e + 1] = __float_as_uint(f.f0[e + 1]) + (__float_as_uint(f.f1[e + 1]) << 9) +
+                   (__float_as_uint(f.f2[e + 1]) << 18) - __float_as_uint(g1) * q.p;
     }
+}
+__device__ __forceinline__ void load_factor(uint32_t (&x)[16], uint32_t tmem, const PrimeK &q) {
+    PlaneSums f;
+    fetch_sums(f, tmem);
+    sums_fetched();
+    combine_planes(x, f, q);
 }
 
 // One forward stage at distance 2^LG in the lane's half rows of NP

@@ -54,7 +54,7 @@ namespace {
 // 1 to 8, polynomials run side by side; one share buffer costs a second
 // cluster barrier), and a pass of the warp kernel with 1, 2 and 3 gates a CTA,
 // per transform slot (k + 2 slots a step).
-constexpr double kTeamStep[3] = {14.5, 16.8, 23.5}, kOneBuffer = 2.5, kWarpSlot[3] = {6.8, 9.8, 11.5};
+constexpr double kTeamStep[3] = {14.2, 15.7, 19.5}, kOneBuffer = 2.5, kWarpSlot[3] = {6.8, 9.4, 11.0};
 
 double team_cost(const LaunchShape &S, uint32_t count, int t) {
     if (!S.team_cap[t]) return 1e30;

@@ -376,8 +376,8 @@ BootstrapFn pick(const LaunchShape &S) {
     }
     if (S.variant < 0 || S.variant >= kNumVariants || S.form < 0 || S.form > 1) return nullptr;
     // The warp kernel takes the default variant wherever it can run (N = 1024, base 2^8, d = 3): at every
-    // measured count it beats variant 2's own kernel (4096 gates, k = 2: 224 against 347 ms; one gate per SM:
-    // 15 against 31 ms), which keeps the other shapes.
+    // measured count it beats variant 2's own kernel (4096 gates, k = 2: 211 against 347 ms; one gate per SM:
+    // 14 against 31 ms), which keeps the other shapes.
     if (S.variant == 2 && warp_form_supported(S)) return launch_bootstrap_warp;
     // At N = 256 the small kernel does, at every measured count (figures in mk_bootstrap_small.cuh).
     if (S.variant == 2 && small_form_supported(S)) return launch_bootstrap_small;
