@@ -288,6 +288,7 @@ struct CircuitPlan {
     cudaGraphExec_t graph = nullptr;
     int graph_form = -1, graph_variant = -1;
     uint32_t graph_cluster = 0;
+    int graph_cluster_mode = -1;
     DeviceKeys graph_keys{};
     ~CircuitPlan() {
         if (graph) cudaGraphExecDestroy(graph);

@@ -560,6 +560,7 @@ void capture_levels(mk_ctx *c, CircuitPlan *pl, const LaunchShape &S, const Devi
         pl->graph_form = c->form;
         pl->graph_variant = c->variant;
         pl->graph_cluster = S.cluster_max;
+        pl->graph_cluster_mode = S.cluster_mode;
         pl->graph_keys = K;
     }
 }
@@ -609,7 +610,7 @@ int run_circuit(mk_ctx *c, int op, uint32_t k, const uint32_t *d_a, const uint32
     // runs launch directly.
     if (e == cudaSuccess && !replayed && c->use_graphs && !c->timing && c->form != MK_FORM_TC) {
         if (pl->graph && (pl->graph_form != c->form || pl->graph_variant != c->variant ||
-                          pl->graph_cluster != S.cluster_max ||
+                          pl->graph_cluster != S.cluster_max || pl->graph_cluster_mode != S.cluster_mode ||
                           std::memcmp(&pl->graph_keys, &K, sizeof(K)) != 0)) {
             cudaGraphExecDestroy(pl->graph);
             pl->graph = nullptr;
