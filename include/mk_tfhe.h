@@ -120,7 +120,9 @@ int mk_ctx_set_batch(mk_ctx *ctx, uint32_t max_gates_per_launch);
  * polynomials per CTA (k <= 8); MK_CLUSTER_AUTO (default) takes the form, and
  * the polynomials per CTA, that the launch's number of gates makes fastest
  * (waves of the gates the device can hold at once, queried when the keys are
- * laid out, times a measured time per wave).  Under MK_FORM_NTT2 at N = 256
+ * laid out, times a measured time per wave); between it and the batched
+ * kernel, AUTO gives variant 2's launches of k >= 2 a kernel with one CTA per
+ * gate where that is the fastest.  Under MK_FORM_NTT2 at N = 256
  * with bg_bit 8 AUTO never takes it (variant 2 is faster).  Other shapes of the
  * NTT forms:
  * one polynomial per CTA, k <= 7; AUTO uses it for launches of at most

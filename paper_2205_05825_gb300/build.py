@@ -29,7 +29,7 @@ BRC_SOURCE = "mk_brc.cu"
 BRC_INSTANCES = [(logn, f) for logn in (8, 10) for f in (0, 1)]
 CPP_SOURCES = ["mk_host.cpp", "mk_circuits.cpp", "mk_server.cpp"]
 HEADERS = ["mk_internal.h", "mk_ctx.h", "mk_bootstrap.cuh", "mk_bulk.cuh", "mk_bootstrap_fft.cuh", "mk_bootstrap_cluster.cuh",
-           "mk_bootstrap_staged.cuh", "mk_bootstrap_split.cuh", "mk_netlist.cuh", "mk_bootstrap_warp.cuh", "mk_bootstrap_team.cuh", "mk_bootstrap_small.cuh",
+           "mk_bootstrap_staged.cuh", "mk_bootstrap_split.cuh", "mk_netlist.cuh", "mk_bootstrap_warp.cuh", "mk_bootstrap_team.cuh", "mk_bootstrap_shared.cuh", "mk_bootstrap_small.cuh",
            BR_SOURCE, BRC_SOURCE]
 
 

@@ -1,5 +1,6 @@
-// Warp and team blind rotations (mk_bootstrap_warp.cuh, mk_bootstrap_team.cuh):
+// Warp, team, shared and N = 256 blind rotations (mk_bootstrap_warp.cuh, _team, _shared, _small):
 // instantiation, launch, and which of them a launch gets.
+#include "mk_bootstrap_shared.cuh"
 #include "mk_bootstrap_small.cuh"
 #include "mk_bootstrap_team.cuh"
 
@@ -55,6 +56,8 @@ namespace {
 // cluster barrier), and a pass of the warp kernel with 1, 2 and 3 gates a CTA,
 // per transform slot (k + 2 slots a step).
 constexpr double kTeamStep[3] = {14.2, 15.7, 19.5}, kOneBuffer = 2.5, kWarpSlot[3] = {6.8, 9.4, 11.0};
+// A pass of the shared kernel (a gate per SM), k = 2 to 8.
+constexpr double kSharedStep[7] = {19.2, 21.3, 27.2, 29.3, 31.9, 38.1, 40.2};
 
 double team_cost(const LaunchShape &S, uint32_t count, int t) {
     if (!S.team_cap[t]) return 1e30;
@@ -69,7 +72,34 @@ double warp_cost(const LaunchShape &S, uint32_t count, uint32_t sms) {
     return (S.k + 2) * ((count / pass) * kWarpSlot[g - 1] + (rest ? kWarpSlot[(rest - 1) / sms] : 0.0));
 }
 
-// The team kernel's teams a CTA for this launch, less one; -1: not its launch.
+bool shared_form_supported(const LaunchShape &S) {
+    return warp_form_supported(S) && S.k >= 2 && br::shared_layout(S.k, S.n).total <= kWarpSmemMax;
+}
+
+// The shared kernel is the default variant's: it runs batches that the batched variants would.
+double shared_cost(const LaunchShape &S, uint32_t count, uint32_t sms) {
+    if (S.variant != 2 || !shared_form_supported(S) || S.k > 8) return 1e30;
+    return kSharedStep[S.k - 2] * ((count + sms - 1) / sms);
+}
+
+cudaError_t launch_bootstrap_shared(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
+                                    const uint32_t *ct_a, const uint32_t *ct_b, const uint32_t *abar_in,
+                                    int64_t max_steps, uint32_t *ext, uint32_t *acc_out, uint32_t count,
+                                    cudaStream_t st) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const size_t smem = br::shared_layout(S.k, S.n).total;
+    auto kern = br::bootstrap_shared_kernel;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const uint32_t grid = count < (uint32_t)sms ? count : (uint32_t)sms;
+    kern<<<grid, 384, smem, st>>>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count);
+    return cudaGetLastError();
+}
+
+// The team kernel's teams a CTA for this launch, less one; 3: the shared kernel; -1: the warp kernel's launch.
 int team_choice(const LaunchShape &S, uint32_t count) {
     if (S.cluster_mode == MK_CLUSTER_OFF || !warp_form_supported(S)) return -1;
     int best = 0;
@@ -81,7 +111,9 @@ int team_choice(const LaunchShape &S, uint32_t count) {
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return -1;
-    return team_cost(S, count, best) < warp_cost(S, count, (uint32_t)sms) ? best : -1;
+    const double team = team_cost(S, count, best), shared = shared_cost(S, count, (uint32_t)sms);
+    if (shared < team && shared < warp_cost(S, count, (uint32_t)sms)) return 3;
+    return team < warp_cost(S, count, (uint32_t)sms) ? best : -1;
 }
 }  // namespace
 
@@ -97,6 +129,7 @@ cudaError_t launch_bootstrap_team(const LaunchShape &S, const DeviceKeys &K, con
         case 0: return br::launch_team<1>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count, st);
         case 1: return br::launch_team<2>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count, st);
         case 2: return br::launch_team<3>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count, st);
+        case 3: return launch_bootstrap_shared(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count, st);
         default: return cudaErrorInvalidConfiguration;
     }
 }

@@ -1,0 +1,43 @@
+"""The shared kernel (two-prime blind rotation at N = 1024, base 2^8: a gate a
+CTA, its polynomials shared out among three teams) against the general
+kernel, word for word, at counts where the launch rule takes it.
+
+Every party count it can take, a part-filled and an over-filled chip, step
+limits inside a party, skipped steps and a party whose steps are all skipped."""
+import numpy as np
+import pytest
+
+from paper_2205_05825_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _abar(P, count, seed):
+    r = np.random.default_rng(seed)
+    abar = r.integers(0, 2 * P["N"], size=(count, P["k"] * P["n"] + 1))
+    abar[r.random(abar.shape) < 0.1] = 0
+    abar[0, :4] = [0, 1, P["N"], 2 * P["N"] - 1]
+    abar[1, :P["n"]] = 0
+    return abar.astype(np.int32)
+
+
+@pytest.mark.parametrize("k,count,steps", [(3, 150, -1), (4, 100, -1), (4, 152, 61), (5, 100, -1), (6, 100, 37), (7, 100, -1),
+                                           (8, 96, -1), (8, 304, 50)])
+def test_accumulators_equal_the_general_kernel(k, count, steps):
+    import torch
+    from paper_2205_05825_gb300 import binding as B
+    P = dict(W.full_params(k), n=24)
+    ctx = B.Context(P, W.CRS_SEED, device=0)
+    for p, s in enumerate(W.party_seeds(k)):
+        ctx.keygen(p, s)
+    dev = torch.from_numpy(_abar(P, count, 10 * k + count)).cuda()
+    accs = []
+    for mode, variant in (("auto", 2), ("off", 0)):
+        acc = torch.full((count, (k + 1) * P["N"]), -1, dtype=torch.int32, device="cuda")
+        ctx.set_cluster(mode)
+        ctx.set_variant(variant)
+        ctx.stage_blind_rotate(dev, steps, acc)
+        ctx.sync()
+        accs.append(acc)
+    assert torch.equal(*accs)
+    ctx.close()
