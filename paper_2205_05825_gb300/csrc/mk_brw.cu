@@ -99,23 +99,64 @@ cudaError_t launch_bootstrap_shared(const LaunchShape &S, const DeviceKeys &K, c
     return cudaGetLastError();
 }
 
-// The team kernel's teams a CTA for this launch, less one; 3: the shared kernel; -1: the warp kernel's launch.
-int team_choice(const LaunchShape &S, uint32_t count) {
-    if (S.cluster_mode == MK_CLUSTER_OFF || !warp_form_supported(S)) return -1;
-    int best = 0;
-    for (int t = 1; t < 3; ++t)
-        if (team_cost(S, count, t) < team_cost(S, count, best)) best = t;
-    if (!S.team_cap[best]) return -1;
-    if (S.cluster_mode == MK_CLUSTER_ON) return best;
+// The fastest kernel for this launch: the team kernel's teams a CTA, less one; 3: the shared kernel; -1: the warp
+// kernel.
+int fastest(const LaunchShape &S, uint32_t count, uint32_t sms, double &cost) {
+    int best = -1;
+    cost = warp_cost(S, count, sms);
+    for (int t = 0; t < 4; ++t) {
+        const double c = t < 3 ? team_cost(S, count, t) : shared_cost(S, count, sms);
+        if (c < cost) cost = c, best = t;
+    }
+    return best;
+}
+
+uint32_t sm_count() {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return -1;
-    const double team = team_cost(S, count, best), shared = shared_cost(S, count, (uint32_t)sms);
-    if (shared < team && shared < warp_cost(S, count, (uint32_t)sms)) return 3;
-    return team < warp_cost(S, count, (uint32_t)sms) ? best : -1;
+        return 0;
+    return (uint32_t)sms;
+}
+
+// The kernel of this launch, as `fastest` numbers them.
+int team_choice(const LaunchShape &S, uint32_t count) {
+    if (S.cluster_mode == MK_CLUSTER_OFF || !warp_form_supported(S)) return -1;
+    if (S.cluster_mode == MK_CLUSTER_ON) {
+        int best = 0;
+        for (int t = 1; t < 3; ++t)
+            if (team_cost(S, count, t) < team_cost(S, count, best)) best = t;
+        return S.team_cap[best] ? best : -1;
+    }
+    const uint32_t sms = sm_count();
+    double cost;
+    return sms ? fastest(S, count, sms, cost) : -1;
 }
 }  // namespace
+
+// A launch whose last pass would leave much of the chip idle: how many of its
+// gates to run first, whole passes of a gate per SM each, so that the rest can
+// have the kernel that is fastest for so few (0: all in one launch).  Two
+// launches in turn cost their sum; 4 % covers the second's start.  Measured
+// (GB300, blind rotation), one launch -> two: k = 2, 200 gates 19.8 -> 18.7 ms, 457 39.0 -> 30.0; k = 4, 200 58.6 -> 49.9,
+// 465 116 -> 84.7, 1001 184 -> 169.6; k = 8, 200 174 -> 155.
+uint32_t bootstrap_head(const LaunchShape &S, uint32_t count) {
+    if (S.cluster_mode != MK_CLUSTER_AUTO || S.variant != 2 || !warp_form_supported(S) || S.k > 8 ||
+        !(S.team_cap[0] | S.team_cap[1] | S.team_cap[2]))
+        return 0;
+    const uint32_t sms = sm_count();
+    if (sms == 0 || count <= sms) return 0;
+    double whole, first, rest;
+    fastest(S, count, sms, whole);
+    double best = 0.96 * whole;
+    uint32_t head = 0;
+    for (uint32_t h = sms; h < count; h += sms) {
+        fastest(S, h, sms, first);
+        fastest(S, count - h, sms, rest);
+        if (first + rest < best) best = first + rest, head = h;
+    }
+    return head;
+}
 
 bool team_form_chosen(const LaunchShape &S, uint32_t count) { return team_choice(S, count) >= 0; }
 

@@ -169,6 +169,7 @@ cudaError_t launch_bootstrap_team(const LaunchShape &S, const DeviceKeys &K, con
 // Whether launch_bootstrap_team takes a launch of `count` gates (its mode, and
 // under MK_CLUSTER_AUTO whether it is the faster form).
 bool team_form_chosen(const LaunchShape &S, uint32_t count);
+uint32_t bootstrap_head(const LaunchShape &S, uint32_t count);
 
 // The two-prime form at N = 256, d = 3, bg_bit = 8 (mk_bootstrap_small.cuh):
 // one CTA a gate, one warp per polynomial and prime.

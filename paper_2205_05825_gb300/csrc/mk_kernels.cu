@@ -408,26 +408,39 @@ int cluster_capacity(const LaunchShape &S) {
     return 0;
 }
 
+namespace {
+// The blind rotation of a launch's gates (NTT and FFT forms), in one or two launches (bootstrap_head).
+cudaError_t launch_gates(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc, const uint32_t *ct_a,
+                         const uint32_t *ct_b, const uint32_t *abar, int64_t max_steps, uint32_t *ext, uint32_t *acc,
+                         uint32_t count, cudaStream_t st) {
+    const uint32_t head = bootstrap_head(S, count);
+    for (uint32_t at = 0, n = head ? head : count; at < count; at += n, n = count - at) {
+        BootstrapFn f = pick_cluster(S, n);
+        if (!f) f = pick(S);
+        if (!f) return cudaErrorInvalidValue;
+        const size_t words = (size_t)S.k * S.N;
+        const cudaError_t e = f(S, K, desc ? desc + at : nullptr, ct_a, ct_b,
+                                abar ? abar + at * ((size_t)S.k * S.n + 1) : nullptr, max_steps,
+                                ext ? ext + at * (words + 1) : nullptr, acc ? acc + at * (words + S.N) : nullptr, n, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+}  // namespace
+
 cudaError_t launch_bootstrap_ntt(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
                                  const uint32_t *ct_a, const uint32_t *ct_b, uint32_t *ext, uint32_t count,
                                  cudaStream_t st) {
     if (count == 0) return cudaSuccess;
     if (S.form == MK_FORM_TC) return launch_bootstrap_tc(S, K, desc, ct_a, ct_b, nullptr, -1, ext, nullptr, count, st);
-    if (BootstrapFn fc = pick_cluster(S, count)) return fc(S, K, desc, ct_a, ct_b, nullptr, -1, ext, nullptr, count, st);
-    BootstrapFn f = pick(S);
-    if (!f) return cudaErrorInvalidValue;
-    return f(S, K, desc, ct_a, ct_b, nullptr, -1, ext, nullptr, count, st);
+    return launch_gates(S, K, desc, ct_a, ct_b, nullptr, -1, ext, nullptr, count, st);
 }
 
 cudaError_t launch_blind_rotate_ntt(const LaunchShape &S, const DeviceKeys &K, const uint32_t *abar,
                                     uint32_t count, int64_t max_steps, uint32_t *acc, cudaStream_t st) {
     if (count == 0) return cudaSuccess;
     if (S.form == MK_FORM_TC) return launch_bootstrap_tc(S, K, nullptr, nullptr, nullptr, abar, max_steps, nullptr, acc, count, st);
-    if (BootstrapFn fc = pick_cluster(S, count))
-        return fc(S, K, nullptr, nullptr, nullptr, abar, max_steps, nullptr, acc, count, st);
-    BootstrapFn f = pick(S);
-    if (!f) return cudaErrorInvalidValue;
-    return f(S, K, nullptr, nullptr, nullptr, abar, max_steps, nullptr, acc, count, st);
+    return launch_gates(S, K, nullptr, nullptr, nullptr, abar, max_steps, nullptr, acc, count, st);
 }
 
 cudaError_t launch_netlist(const LaunchShape &S, const DeviceKeys &K, const NetlistArgs &A, uint32_t sm_count,
