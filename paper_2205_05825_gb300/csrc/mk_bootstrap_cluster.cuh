@@ -1,5 +1,8 @@
 // mk_bootstrap_cluster.cuh -- the latency form of the blind rotation: one
-// thread-block cluster per gate, one CTA per accumulator polynomial.
+// thread-block cluster per gate, one CTA per accumulator polynomial.  It runs
+// the Goldilocks form, base 2^8 with other N or d, other bases, and N = 256
+// where the latency form is forced; two-prime launches at N = 1024, base 2^8
+// take mk_bootstrap_team.cuh.
 //
 // The batched kernel (mk_bootstrap.cuh) gives each gate one CTA, which runs
 // the (k+2)(d+1) transforms of every CMux step one after the other.  For a

@@ -24,7 +24,8 @@
 // gates on the chip at once.  Measured (GB300, blind rotation of one wave):
 // k = 2: 1 gate 6.4 ms (the cluster kernel it replaces 11.5, the warp kernel
 // 15.7), 37 gates 7.7, 76 gates (T = 2) 8.4, 152 gates (T = 3) 10.7 against 14.3;
-// k = 4: 1 gate 13.3 (23.7), 5 gates 13.5; k = 8: 1 gate 36 ms against 150.
+// k = 4: 1 gate 13.3 (23.7), 5 gates 13.5; k = 8: 1 gate 34 ms against 150.
+// From about 77 gates the shared kernel (mk_bootstrap_shared.cuh) is faster.
 // A step is a chain of dependent phases: at T = 1 about 11.8 k clocks, of them
 // digits 0.6, two products 0.8 each, two sets of butterflies and key products
 // 2.3 and 1.9, the cluster barrier 1.0, two inverse transforms 1.4 each.

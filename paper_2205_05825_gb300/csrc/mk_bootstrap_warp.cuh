@@ -44,8 +44,8 @@
 // the register file, and its fragments need a transposition.)
 //
 // Measured (GB300, whole blind rotation): 4096 gates at k = 2 347 -> 211 ms,
-// 1001 at k = 4 308 -> 182 ms, 96 at k = 8 333 -> 139 ms, 152 at k = 2 (one gate
-// per SM) 31 -> 14.3 ms.  Per CMux step and gate 23.7 -> 14.5 k clocks of an SM;
+// 1001 at k = 4 308 -> 184 ms (170 with the last pass in another kernel,
+// bootstrap_head), 152 at k = 2 (one gate per SM) 31 -> 14.3 ms.  Per CMux step and gate 23.7 -> 14.5 k clocks of an SM;
 // the multiply pipe is 81 % busy (ncu, three gates an SM).
 //
 // A CTA holds G gates (4 G warps) and the tables once; the grid is at most one

@@ -352,6 +352,7 @@ struct mk_ctx {
     size_t bk_words() const { return (size_t)P.n * 3 * P.d * P.N; }
     size_t ks_words() const { return (size_t)P.N * P.t * ((1u << P.ks_bit) - 1) * (P.n + 1); }
     LaunchShape shape() const {
+        // Shapes that the team kernel does not take (mk_brw.cu has its rule).
         // AUTO: the cluster kernel while the launch's gates fit in max(1,
         // floor(k/2)) waves of resident clusters (cluster_cap, queried from
         // the device for the form's kernel); beyond that the batched kernel's

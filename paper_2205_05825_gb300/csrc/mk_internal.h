@@ -73,7 +73,8 @@ struct LaunchShape {
     int variant;  // blind-rotation variant (see kVariantNpf)
     int form;     // MK_FORM_*
     // Batches of at most this many gates run the cluster (latency) kernel of
-    // the NTT forms: one CTA per accumulator polynomial (0: never).
+    // the NTT forms: one CTA per accumulator polynomial (0: never).  Shapes
+    // of the warp kernel take the team kernel instead (below).
     uint32_t cluster_max;
     // Latency forms of the warp kernel's shapes: MK_CLUSTER_* and, per teams a
     // CTA (1, 2, 3), the gates resident at once (team_capacities).
