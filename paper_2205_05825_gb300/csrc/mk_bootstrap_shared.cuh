@@ -152,7 +152,8 @@ bootstrap_shared_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict_
     uint32_t phase = 0, vphase = 0;               // products waited for
     bool reading = false;                         // team 2: a step's shares may still be being read
 
-    // The digits of (X^-e - 1) ACC_jj, and one thread's issue of a product of the digits stored.
+    // The digits of (X^-e - 1) ACC_jj, and the issue of their products by an elected lane (lane 0: 152 gates at
+    // k = 4 31.4 against 30.1 ms).
     auto cut_digits = [&](int jj, uint32_t e) {
         const uint32_t *ap = acc + jj * N;
         uint32_t w[8];
