@@ -27,14 +27,13 @@
 // kernel's rate with three gates side by side: the multiply pipe bounds it, and
 // for few parties the chain of phase B does.
 //
-// Hand-over (each a named barrier, so the one who gives does not wait):
+// Hand-over, by named barriers (at 4 and 7 the one who gives does not wait):
 //   4: teams 1 and 2 have stored their shares; team 0 waits.
-//   7: team 0 has read them; team 2 waits before it stores the next step's
-//      (team 1 has by then seen v's products, which come after the reading).
-//   6: team 1 has read v's products; team 0 waits before its columns are used
-//      again.
-// v's products have an mbarrier of their own, one phase a step: team 1 is never
-// more than one phase behind or ahead, because step s + 1's need its share.
+//   7: team 0 has read them; team 2 waits before it stores the next step's.
+//   6: teams 0 and 1 have read v's products; both wait, so team 1 is never a
+//      step ahead of team 0 whatever became of a wait for products: without
+//      that it would arrive at 4 twice after a wait that ran out.
+// v's products have an mbarrier of their own, one phase a step.
 // Where the party changes the polynomials change hands: all teams meet (9).
 // Waits for products are bounded (products_wait) and nothing branches on their
 // outcome, so no team misses a barrier.
@@ -248,10 +247,7 @@ bootstrap_shared_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict_
                 }
                 if (last) {
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                    if (team == 1)
-                        asm volatile("bar.arrive 6, 256;\n" ::: "memory");
-                    else
-                        asm volatile("bar.sync 6, 256;\n" ::: "memory");
+                    asm volatile("bar.sync 6, 256;\n" ::: "memory");
                 }
                 // the next slot's products run under this one's butterflies
                 const bool same = s + 1 < slots;

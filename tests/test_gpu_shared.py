@@ -5,7 +5,8 @@ that run as two launches.
 
 Every party count it can take, a part-filled and an over-filled chip, step
 limits inside a party, skipped steps and a party whose steps are all skipped;
-gates whose last pass has one gate, some, and nearly all of the chip."""
+gates whose last pass has one gate, some, and nearly all of the chip; and the
+bounded wait."""
 import numpy as np
 import pytest
 
@@ -68,4 +69,25 @@ def test_gates_of_two_launches_equal_the_general_kernel(k, count):
         ctx.sync()
         outs.append(out)
     assert torch.equal(*outs)
+    ctx.close()
+
+
+def test_products_wait_runs_out_and_the_context_recovers():
+    import torch
+    from paper_2205_05825_gb300 import binding as B
+    P = dict(W.full_params(4), n=24)
+    ctx = _ctx(P)
+    dev = torch.from_numpy(_abar(P, 100, 5)).cuda()
+    good, acc = (torch.zeros((100, 5 * P["N"]), dtype=torch.int32, device="cuda") for _ in range(2))
+    ctx.stage_blind_rotate(dev, -1, good)
+    ctx.sync()
+    step = int(np.flatnonzero(dev[0, :24].cpu().numpy())[3])
+    ctx.debug_fault("skip_key_step", step, 20_000_000)
+    ctx.stage_blind_rotate(dev, -1, acc)
+    with pytest.raises(B.MkError, match="MK_ETIMEOUT"):
+        ctx.sync()
+    ctx.debug_fault("none")
+    ctx.stage_blind_rotate(dev, -1, acc)
+    ctx.sync()
+    assert torch.equal(acc, good)
     ctx.close()
