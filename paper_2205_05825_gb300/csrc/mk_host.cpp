@@ -417,10 +417,14 @@ int ensure_device_keys(mk_ctx *c) {
             c->d_ksp = nullptr;  // no room: the key switch runs its kernels on the plain rows
             (void)cudaGetLastError();
         }
-        if (c->d_ksp) {
-            MK_CUDA(c, cudaStreamSynchronize(cudaStreamLegacy));  // the rows have landed
-            MK_CUDA(c, build_keyswitch_planes(c->shape(), c->d_ks, c->d_ksp, c->stream));
-        }
+    }
+    // A copy from pageable memory may return before its data has landed, and the planes are built on the device.
+    // All of it is finished here, once per layout: the next call may come on another stream (mk_ctx_set_stream),
+    // which nothing orders after this one.
+    MK_CUDA(c, cudaStreamSynchronize(cudaStreamLegacy));
+    if (c->d_ksp) {
+        MK_CUDA(c, build_keyswitch_planes(c->shape(), c->d_ks, c->d_ksp, c->stream));
+        MK_CUDA(c, cudaStreamSynchronize(c->stream));
     }
     c->cluster_cap = (uint32_t)cluster_capacity(c->shape());
     team_capacities(c->shape(), c->team_cap);
