@@ -106,7 +106,8 @@ __device__ __forceinline__ void kt_ld16(uint32_t addr, float *r) {
         : "r"(addr));
 }
 
-// grid.x: column tile fastest, then party, then K range; grid.y: group of 128 MT gates.
+// Blocks: column tile fastest, then party, then K range, then group of 128 MT gates (all on grid.x: grid.y would end
+// at 65535 groups, 16.8 M rows).
 template <int MT>
 __global__ void __launch_bounds__(KT_THREADS, 1)
     keyswitch_tc_kernel(LaunchShape S, const unsigned char *__restrict__ planes, const GateDesc *__restrict__ desc,
@@ -117,8 +118,9 @@ __global__ void __launch_bounds__(KT_THREADS, 1)
     uint16_t *words = reinterpret_cast<uint16_t *>(smem + KT_OFF_WORDS);
     const uint32_t n = S.n, N = S.N, k = S.k;
     const uint32_t E = k * N + 1, W = k * n + 1;
-    const uint32_t tile = blockIdx.x % tiles, party = blockIdx.x / tiles % k, split = blockIdx.x / tiles / k;
-    const uint32_t g0 = blockIdx.y * 128 * MT;
+    const uint32_t items = tiles * k * splits, item = blockIdx.x % items;
+    const uint32_t tile = item % tiles, party = item / tiles % k, split = item / tiles / k;
+    const uint32_t g0 = blockIdx.x / items * (128 * MT);
     const uint32_t chunks = N / KT_CHUNK, c0 = split * chunks / splits, c1 = (split + 1) * chunks / splits;
     const uint32_t kb0 = c0 * (KT_CHUNK / 2), nkb = (c1 - c0) * (KT_CHUNK / 2);  // coefficient pairs of this item
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -327,25 +329,26 @@ cudaError_t launch_keyswitch_tc(const LaunchShape &S, const DeviceKeys &K, const
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const uint32_t tiles = column_tiles(S), mt = count > 128 ? 2 : 1, groups = (count + 128 * mt - 1) / (128 * mt);
+    const uint32_t tiles = column_tiles(S), mt = count > 128 ? 2 : 1, groups = (count - 1) / (128 * mt) + 1;
     // K ranges per item: the fewest waves x (a fixed cost of about 8 us + the range's pairs at the slower of the
     // MMAs, 0.19 us per 128 gates, and the key copy, 0.3 us)
     uint32_t splits = 1;
     double best = 1e30;
     for (uint32_t s = 1; s <= S.N / KT_CHUNK; s *= 2) {
-        const uint32_t waves = (tiles * S.k * groups * s + sms - 1) / sms;
-        const double us = waves * (8.0 + (S.N / 2 / s) * (mt == 2 ? 0.38 : 0.3));
+        const uint64_t waves = ((uint64_t)tiles * S.k * groups * s + sms - 1) / sms;
+        const double us = (double)waves * (8.0 + (S.N / 2 / s) * (mt == 2 ? 0.38 : 0.3));
         if (us < best) {
             best = us;
             splits = s;
         }
     }
+    const uint64_t grid = (uint64_t)tiles * S.k * splits * groups;
+    if (grid > 0x7FFFFFFFu || count > 0x7FFFFFFFu) return cudaErrorInvalidConfiguration;  // before any row is written
     keyswitch_init_kernel<<<count, 256, 0, st>>>(S, desc, ext, out);
-    const dim3 grid(tiles * S.k * splits, groups);
     auto run = [&](auto kern) {
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KT_SMEM);
         if (err != cudaSuccess) return err;
-        kern<<<grid, KT_THREADS, KT_SMEM, st>>>(S, static_cast<const unsigned char *>(K.ks_planes), desc, ext, out, count,
+        kern<<<(uint32_t)grid, KT_THREADS, KT_SMEM, st>>>(S, static_cast<const unsigned char *>(K.ks_planes), desc, ext, out, count,
                                                 tiles, splits, K.status);
         return cudaGetLastError();
     };
