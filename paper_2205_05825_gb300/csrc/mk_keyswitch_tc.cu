@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1)
                 kt_commit(empty0 + 8 * st);
             }
             kt_commit(done);  // every MMA of this thread
-            if (!ok) kt_wait(done, 0, KT_DRAIN_NS, nullptr);
+            kt_wait(done, 0, KT_DRAIN_NS, nullptr);  // whatever became of the builders' wait for it
         }
         __syncwarp();
     } else if (warp < 4 * MT) {
