@@ -132,13 +132,16 @@ enum { MK_CLUSTER_AUTO = 0, MK_CLUSTER_OFF = 1, MK_CLUSTER_ON = 2 };
 int mk_ctx_set_cluster(mk_ctx *ctx, int mode);
 
 /* Test hook for the kernels' bounded waits (no paper counterpart).  Every
- * wait of the staged blind rotation (variant 6) for a key copy, of the warp
- * kernel (variant 2) for its matrix products and of the
- * tcgen05 product engine (MK_FORM_TC, variant 1) gives up after wait_ns of
- * global time (0: the default, 1 s); a kernel whose wait gave up stops its
- * work, lets its own copies and tensor-core operations finish, and returns
- * without its outputs; the next mk_sync reports MK_ETIMEOUT, and the context
- * stays usable.  kind MK_FAULT_SKIP_KEY_STEP: until the next call, the staged
+ * wait of the staged blind rotation (variant 6) and of the cluster kernel for
+ * a key copy, of MK_FORM_NTT2's kernels that compute on the tensor cores for
+ * their matrix products, of the matrix-product key switch and of the tcgen05
+ * product engine (MK_FORM_TC) gives up after wait_ns of
+ * global time (0: the default, 1 s).  A kernel whose wait gave up lets its own
+ * copies and tensor-core operations finish before it returns; its outputs are
+ * undefined (the staged kernel, the key switch and the product engine stop
+ * their work; the other blind rotations run through, without further waits, so
+ * that none of their CTAs or warps is left at a barrier).  The next mk_sync
+ * reports MK_ETIMEOUT, and the context stays usable.  kind MK_FAULT_SKIP_KEY_STEP: until the next call, the staged
  * kernel and the cluster latency kernel never copy the key entry of CMux step
  * `arg` (0-based), or, where the latency form computes on the tensor cores,
  * never start that step's products, so the waits for it run out.  kind MK_FAULT_SKIP_DIGIT_TILE: in the next tcgen05

@@ -357,7 +357,9 @@ bootstrap_shared_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict_
         }
         __syncthreads();
     }
-    // every product committed has been waited for (or its wait ran out: bounded above)
+    // no product is in flight when TMEM is freed; the exchange buffers are free since the last __syncthreads
+    if (warp == 0 && elect_one()) products_drain(st_smem_addr(ex), K.status);
+    __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");

@@ -361,6 +361,9 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
             }
         }
     }
+    // no product is in flight when TMEM is freed; a team's exchange buffer is free since its last quad_sync
+    if (warp == 0 && elect_one()) products_drain(st_smem_addr(ex), K.status);
+    __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");

@@ -297,7 +297,8 @@ __device__ __forceinline__ void issue_products(uint32_t tmem, uint32_t d, uint32
 
 // Wait for a gate's products, bounded in global time.  Nothing branches on
 // the outcome: a wait that runs out sets the abort and status words (mk_sync
-// reports MK_ETIMEOUT) and later waits of the CTA return at once.
+// reports MK_ETIMEOUT), later waits of the CTA return at once, and its gates
+// run to their end on whatever TMEM holds: their results are garbage.
 __device__ __noinline__ void products_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort, uint64_t wait_ns,
                                            uint32_t *status) {
     if (*abort) return;
@@ -308,6 +309,26 @@ __device__ __noinline__ void products_wait(uint32_t bar, uint32_t parity, volati
         if (st_globaltimer() - t0 > wait_ns) break;
     }
     *abort = 1u;
+    atomicOr(status, kStatusWarp);
+}
+
+// At a kernel's end, the thread that issued a gate's products: every one of
+// them has completed when this returns, so that TMEM and shared memory can be
+// given back.  After a wait that ran out nothing else says so: later waits
+// return at once, and a barrier that missed a commit is a phase behind.  The
+// bound is this function's own.  bar: eight bytes of shared memory that
+// nothing else uses any more.
+constexpr uint64_t kDrainNs = 1000000000ull;
+__device__ __noinline__ void products_drain(uint32_t bar, uint32_t *status) {
+    st_mbar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    st_fence_proxy_async();
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+    const uint64_t t0 = st_globaltimer();
+    for (uint32_t it = 0; it < (1u << 30); ++it) {
+        if (st_mbar_try(bar, 0)) return;
+        if (st_globaltimer() - t0 > kDrainNs) break;
+    }
     atomicOr(status, kStatusWarp);
 }
 
@@ -817,7 +838,9 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
         }
         quad_sync(bar);
     }
-    // every product committed has been waited for (or its wait ran out: bounded above)
+    // no product is in flight when TMEM is freed; the slot's exchange buffer is free since its last quad_sync
+    if (warp == 0 && lane == 0) products_drain(st_smem_addr(ex), K.status);
+    __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
