@@ -397,7 +397,7 @@ uint32_t team_capacity(uint32_t k, uint32_t n) {
     const size_t smem = team_layout(k, n, T).total;
     if ((k + T) / T > 8 || smem > kWarpSmemMax) return 0;
     auto kern = bootstrap_team_kernel<T>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    if (allow_smem(kern) != cudaSuccess) return 0;
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = team_config<T>(k, n, 1, nullptr, attr);
     int clusters = 0;
@@ -410,8 +410,7 @@ cudaError_t launch_team(const LaunchShape &S, const DeviceKeys &K, const GateDes
                         const uint32_t *ct_b, const uint32_t *abar_in, int64_t max_steps, uint32_t *ext,
                         uint32_t *acc_out, uint32_t count, cudaStream_t st) {
     auto kern = bootstrap_team_kernel<T>;
-    const size_t smem = team_layout(S.k, S.n, T).total;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = team_config<T>(S.k, S.n, count, st, attr);

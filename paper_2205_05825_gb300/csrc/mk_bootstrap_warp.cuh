@@ -169,6 +169,15 @@ __host__ __device__ inline WarpLayout warp_layout(uint32_t k, uint32_t n, uint32
     return L;
 }
 
+// Lets a kernel have all of an SM's shared memory.  The limit is the kernel's,
+// not the launch's: set to what each launch needs, a smaller one from another
+// thread (other gates a CTA, or another context's k and n) could come between
+// a thread's setting and its launch, which would then be refused.
+template <class Kernel>
+cudaError_t allow_smem(Kernel kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWarpSmemMax);
+}
+
 __device__ __forceinline__ void quad_sync(int bar) { asm volatile("bar.sync %0, 128;\n" ::"r"(bar) : "memory"); }
 
 // Accumulator polynomials: coefficient m at m ^ 16 (m / 32 mod 2), so that a

@@ -34,7 +34,7 @@ cudaError_t launch_bootstrap_warp(const LaunchShape &S, const DeviceKeys &K, con
     const uint32_t g = warp_gates(S.k, S.n, count, (uint32_t)sms);
     const size_t smem = br::warp_layout(S.k, S.n, g).total;
     auto kern = br::bootstrap_warp_kernel;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = br::allow_smem(kern);
     if (e != cudaSuccess) return e;
     const uint32_t grid = count < (uint32_t)sms ? count : (uint32_t)sms;
     kern<<<grid, 128 * g, smem, st>>>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count);
@@ -92,7 +92,7 @@ cudaError_t launch_bootstrap_shared(const LaunchShape &S, const DeviceKeys &K, c
     if (e != cudaSuccess) return e;
     const size_t smem = br::shared_layout(S.k, S.n).total;
     auto kern = br::bootstrap_shared_kernel;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = br::allow_smem(kern);
     if (e != cudaSuccess) return e;
     const uint32_t grid = count < (uint32_t)sms ? count : (uint32_t)sms;
     kern<<<grid, 384, smem, st>>>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out, count);
@@ -188,7 +188,7 @@ cudaError_t launch_bootstrap_small(const LaunchShape &S, const DeviceKeys &K, co
     if (!small_form_supported(S) || K.tw_split == nullptr) return cudaErrorInvalidValue;
     const size_t smem = br::small_layout(S.k, S.n).total;
     auto run = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = br::allow_smem(kern);
         if (e != cudaSuccess) return e;
         kern<<<count, 64 * (S.k + 1), smem, st>>>(S, K, desc, ct_a, ct_b, abar_in, max_steps, ext, acc_out);
         return cudaGetLastError();
