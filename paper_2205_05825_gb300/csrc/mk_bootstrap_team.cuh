@@ -391,6 +391,34 @@ cudaLaunchConfig_t team_config(uint32_t k, uint32_t n, uint32_t count, cudaStrea
     return cfg;
 }
 
+// Registers that a CTA takes from its SM (allocated in units of 8 a thread).
+template <int T>
+uint32_t team_registers() {
+    cudaFuncAttributes a;
+    if (cudaFuncGetAttributes(&a, bootstrap_team_kernel<T>) != cudaSuccess) return 0;
+    return (uint32_t)((a.numRegs + 7) / 8 * 8) * 128 * T;
+}
+
+// Whether no SM can hold CTAs of these kernels that want more than its 512
+// TMEM columns together, from one launch or from several streams'.  An
+// allocation waits until columns are free, and a CTA that has its own waits
+// for its cluster: two clusters, each holding an SM's columns that the other
+// asks for, would wait for ever, and occupancy queries know nothing of TMEM.
+// T = 1 (256 columns) may have two CTAs an SM, T = 2 and 3 (512) must be alone
+// among them.  Registers see to it (255, 238 and 168 a thread of 65536); they
+// are the compiler's choice, so they are checked.  (Kernels without clusters
+// only delay each other: whoever holds columns gets to its end.)
+inline bool teams_fit_tmem() {
+    static_assert(Operands<1>::columns == 256 && Operands<2>::columns == 512 && Operands<3>::columns == 512, "TMEM columns");
+    int dev = 0, file = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&file, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess)
+        return false;
+    const uint32_t r1 = team_registers<1>(), r2 = team_registers<2>(), r3 = team_registers<3>(), all = (uint32_t)file;
+    const uint32_t least = r1 < r2 ? (r1 < r3 ? r1 : r3) : (r2 < r3 ? r2 : r3);
+    return 3 * r1 > all && r2 + least > all && r3 + least > all;
+}
+
 // Gates of this shape that can be resident at once, or 0 if none can.
 template <int T>
 uint32_t team_capacity(uint32_t k, uint32_t n) {

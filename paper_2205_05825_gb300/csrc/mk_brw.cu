@@ -43,7 +43,7 @@ cudaError_t launch_bootstrap_warp(const LaunchShape &S, const DeviceKeys &K, con
 
 void team_capacities(const LaunchShape &S, uint32_t cap[3]) {
     cap[0] = cap[1] = cap[2] = 0;
-    if (!warp_form_supported(S)) return;
+    if (!warp_form_supported(S) || !br::teams_fit_tmem()) return;
     cap[0] = br::team_capacity<1>(S.k, S.n);
     cap[1] = br::team_capacity<2>(S.k, S.n);
     cap[2] = br::team_capacity<3>(S.k, S.n);
