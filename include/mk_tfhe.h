@@ -143,15 +143,25 @@ int mk_ctx_set_cluster(mk_ctx *ctx, int mode);
  * that none of their CTAs or warps is left at a barrier).  The next mk_sync
  * reports MK_ETIMEOUT, and the context stays usable.  kind MK_FAULT_SKIP_KEY_STEP: until the next call, the staged
  * kernel and the cluster latency kernel never copy the key entry of CMux step
- * `arg` (0-based), or, where the latency form computes on the tensor cores,
- * never start that step's products, so the waits for it run out.  kind MK_FAULT_SKIP_DIGIT_TILE: in the next tcgen05
+ * `arg` (0-based), and MK_FORM_NTT2's kernels that compute on the tensor
+ * cores (at N = 1024 with bg_bit 8) never start that step's products, so the
+ * waits for it run out.  kind MK_FAULT_SKIP_KEY_TILE: until the next call, the
+ * matrix-product key switch never copies the key tiles of coefficient pair
+ * `arg` (coefficients 2 arg and 2 arg + 1 of every party).  kind
+ * MK_FAULT_SKIP_DIGIT_TILE: in the next tcgen05
  * launch, the first CTA that reaches its digit tile `arg` does not load it
  * (one shot).  kind MK_FAULT_SKIP_WIRE_READY: until the next call, the
  * persistent operator launch never marks the output of its work item `arg`
  * (0-based, in the plan's level order) ready, so once every other gate has
- * finished, the gates that read it give up after the bound.  MK_FAULT_NONE clears all three.  Nothing here
+ * finished, the gates that read it give up after the bound.  MK_FAULT_NONE clears all of them.  Nothing here
  * faults the device: a skipped copy or mark is one that is never issued. */
-enum { MK_FAULT_NONE = 0, MK_FAULT_SKIP_KEY_STEP = 1, MK_FAULT_SKIP_DIGIT_TILE = 2, MK_FAULT_SKIP_WIRE_READY = 3 };
+enum {
+    MK_FAULT_NONE = 0,
+    MK_FAULT_SKIP_KEY_STEP = 1,
+    MK_FAULT_SKIP_DIGIT_TILE = 2,
+    MK_FAULT_SKIP_WIRE_READY = 3,
+    MK_FAULT_SKIP_KEY_TILE = 4
+};
 int mk_debug_fault(mk_ctx *ctx, int kind, int64_t arg, uint64_t wait_ns);
 
 /* The k-bit operators evaluate their netlist level by level.  With graphs on

@@ -246,7 +246,8 @@ class Context:
         """Latency (cluster) kernel: "auto" (small launches), "on" or "off"."""
         self._check(self.L.mk_ctx_set_cluster(self.h, CLUSTER_MODES[mode]), "mk_ctx_set_cluster")
 
-    FAULTS = {"none": 0, "skip_key_step": 1, "skip_digit_tile": 2, "skip_wire_ready": 3}
+    FAULTS = {"none": 0, "skip_key_step": 1, "skip_digit_tile": 2, "skip_wire_ready": 3,
+              "skip_key_tile": 4}
     CIRCUIT_EXEC = {"auto": 0, "levels": 1, "persistent": 2}
 
     def set_circuit_exec(self, mode):
@@ -255,8 +256,8 @@ class Context:
         self._check(self.L.mk_ctx_set_circuit_exec(self.h, self.CIRCUIT_EXEC[mode]), "mk_ctx_set_circuit_exec")
 
     def debug_fault(self, kind="none", arg=0, wait_ns=0):
-        """Test hook of the bounded waits (mk_debug_fault): skip one key copy
-        of the staged kernel or one digit tile of the tcgen05 engine."""
+        """Test hook of the bounded waits (mk_debug_fault): withhold one step's
+        key copy or matrix products, one digit or key tile, or one wire."""
         self._check(self.L.mk_debug_fault(self.h, self.FAULTS[kind], int(arg), int(wait_ns)), "mk_debug_fault")
 
     def set_graphs(self, on):

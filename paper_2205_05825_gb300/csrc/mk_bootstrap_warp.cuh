@@ -709,11 +709,11 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
             }
             store_digits(unit, w);
         };
-        auto start_products = [&]() {
+        auto start_products = [&](bool issue) {
             st_fence_proxy_async();
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             quad_sync(bar);
-            if (warp == 0 && lane == 0) {
+            if (warp == 0 && lane == 0 && issue) {
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 issue_products<kWarpMaxGates>(ctl->tmem, tmem, ones_s, plane0_s, digits_s, mbar);
             }
@@ -732,6 +732,7 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
         for (int step = next_step(0); step < limit; step = next) {
             const int i = step / n + 1;
             const uint32_t e = abar[step];
+            const bool issue = step != S.skip_key_step;
             next = next_step(step + 1);
             const uint4 *bk = bk_all + (size_t)step * 9 * POLY + pr * (POLY / 2);
             uint32_t V[16];
@@ -739,7 +740,7 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
             for (int c = 0; c < 16; ++c) V[c] = 0;
             if (!started) {
                 cut_digits(poly_of(0, i), e);
-                start_products();
+                start_products(issue);
             }
             // The next step's first slot can start in this step's last one if its polynomial is final by then:
             // another party's, so not one of this step's 0 and i.
@@ -758,7 +759,7 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
                 // the next slot's products run under this one's butterflies
                 if (s < k || (s == k + 1 && started)) {
                     cut_digits(s < k ? poly_of(s + 1, i) : poly_of(0, i), s < k ? e : abar[next]);
-                    start_products();
+                    start_products(s < k ? issue : next != S.skip_key_step);
                 }
                 // R1 = <x, key1>, R2 = <x, key2> in place of x[0], x[1]: (d, A_jj), or (f0, f1) of v's digits
                 const uint4 *k1 = bk + (s <= k ? 0 : 3 * POLY);
@@ -825,7 +826,7 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
 #pragma unroll
                         for (int c = 0; c < 8; ++c) z[c] += gad.offset;
                         store_digits(unit, z);
-                        start_products();
+                        start_products(issue);
                     } else {
                         uint32_t *ap = acc + (s == k + 1 ? (job ? i : 0) : jj) * N;
 #pragma unroll

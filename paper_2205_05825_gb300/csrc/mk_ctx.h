@@ -324,7 +324,8 @@ struct mk_ctx {
     void *d_ksp = nullptr;      // key-switching keys as matrix operands (mk_keyswitch_tc.cu), if supported
     uint32_t *d_status = nullptr;  // status word of the kernels' bounded waits (bit 0: one ran out)
     uint64_t wait_ns = 1000000000ull;  // bound on each such wait (1 s)
-    int64_t debug_skip_key_step = -1;  // test hook of the staged kernel (see LaunchShape)
+    int64_t debug_skip_key_step = -1;  // test hooks of the bounded waits (see LaunchShape)
+    int64_t debug_skip_key_tile = -1;
     void *d_tcws = nullptr;     // MK_FORM_TC wave workspace for tc_ws_gates gates
     uint32_t tc_ws_gates = 0;
     uint32_t *d_ext = nullptr;  // scratch [scratch_gates][k*N+1]
@@ -366,7 +367,8 @@ struct mk_ctx {
                               : cluster_mode == MK_CLUSTER_OFF ? 0u
                                                                : waves * cluster_cap;
         return LaunchShape{P.n, P.N, logN, P.k, P.d, P.bg_bit, P.ks_bit, P.t, variant, form, cmax,
-                           cluster_mode, {team_cap[0], team_cap[1], team_cap[2]}, wait_ns, debug_skip_key_step};
+                           cluster_mode, {team_cap[0], team_cap[1], team_cap[2]}, wait_ns, debug_skip_key_step,
+                           debug_skip_key_tile};
     }
     DeviceKeys dkeys() const {
         // twiddles: [2][N] of 8-byte (NTT) or 16-byte (NTT2) entries; FFT: one [3][N/2] table

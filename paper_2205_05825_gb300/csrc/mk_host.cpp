@@ -818,13 +818,14 @@ int mk_ctx_set_cluster(mk_ctx *c, int mode) {
 int mk_debug_fault(mk_ctx *c, int kind, int64_t arg, uint64_t wait_ns) {
     if (!c) return MK_EINVAL;
     if (kind != MK_FAULT_NONE && kind != MK_FAULT_SKIP_KEY_STEP && kind != MK_FAULT_SKIP_DIGIT_TILE &&
-        kind != MK_FAULT_SKIP_WIRE_READY)
+        kind != MK_FAULT_SKIP_WIRE_READY && kind != MK_FAULT_SKIP_KEY_TILE)
         return fail(c, MK_EINVAL, "unknown fault kind");
     if (kind != MK_FAULT_NONE && arg < 0) return fail(c, MK_EINVAL, "fault argument must be >= 0");
     c->debug_skip_item = kind == MK_FAULT_SKIP_WIRE_READY ? arg : -1;
     if (kind == MK_FAULT_SKIP_DIGIT_TILE && c->device < 0) return fail(c, MK_EDEVICE, "host-only context");
     c->wait_ns = wait_ns ? wait_ns : 1000000000ull;
     c->debug_skip_key_step = kind == MK_FAULT_SKIP_KEY_STEP ? arg : -1;
+    c->debug_skip_key_tile = kind == MK_FAULT_SKIP_KEY_TILE ? arg : -1;
     if (c->device >= 0) {
         MK_CUDA(c, cudaSetDevice(c->device));
         MK_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -85,6 +85,9 @@ struct LaunchShape {
     // issued, so the waits for them run out (-1: none).
     uint64_t wait_ns;
     int64_t skip_key_step;
+    // The same for the matrix-product key switch: this coefficient pair's key
+    // tiles (of every party) are never copied (-1: none).
+    int64_t skip_key_tile;
 };
 
 // Clusters of the latency form that fit on the device at once for this

@@ -161,11 +161,12 @@ __global__ void __launch_bounds__(KT_THREADS, 1)
                     ok = false;
                     break;
                 }
+                if (kb0 + kb == S.skip_key_tile) continue;  // test hook
                 st_bulk_load(stage0 + st * KT_STAGE, src + (size_t)kb * tiles * KT_BBLOCK, KT_BBLOCK, full0 + 8 * st);
             }
             // no copy may be in flight when the CTA exits
             for (uint32_t q = kb > KT_STAGES ? kb - KT_STAGES : 0; q < kb; ++q)
-                kt_wait(full0 + 8 * (q % KT_STAGES), (q / KT_STAGES) & 1, KT_DRAIN_NS, nullptr);
+                if (kb0 + q != S.skip_key_tile) kt_wait(full0 + 8 * (q % KT_STAGES), (q / KT_STAGES) & 1, KT_DRAIN_NS, nullptr);
         }
         __syncwarp();
     } else if (warp == 9) {
