@@ -321,6 +321,7 @@ struct mk_ctx {
     uint64_t *d_bk = nullptr;   // [k][n][3][d][N]
     uint64_t *d_keyA = nullptr; // [(k+1)][d][N]
     uint32_t *d_ks = nullptr;   // [k][N][t][B'-1][n+1]
+    void *d_warp = nullptr;     // the warp kernel's tables (MK_FORM_NTT2 at N = 1024)
     void *d_ksp = nullptr;      // key-switching keys as matrix operands (mk_keyswitch_tc.cu), if supported
     uint32_t *d_status = nullptr;  // status word of the kernels' bounded waits (bit 0: one ran out)
     uint64_t wait_ns = 1000000000ull;  // bound on each such wait (1 s)
@@ -374,7 +375,7 @@ struct mk_ctx {
         // twiddles: [2][N] of 8-byte (NTT) or 16-byte (NTT2) entries; FFT: one [3][N/2] table
         const size_t half = (form == MK_FORM_NTT2 ? 16 : (form == MK_FORM_FFT ? 0 : 8)) * (size_t)P.N;
         const void *split = form == MK_FORM_NTT2 ? (const unsigned char *)d_tw + 32 * (size_t)P.N : nullptr;
-        const void *warp = form == MK_FORM_NTT2 && P.N == 1024 ? (const unsigned char *)d_tw + 64 * (size_t)P.N : nullptr;
+        const void *warp = form == MK_FORM_NTT2 ? d_warp : nullptr;
         return DeviceKeys{d_tw, (const unsigned char *)d_tw + half, d_bk, d_keyA, d_ks, d_tcws, tc_ws_gates, d_status,
                           split, warp, d_ksp};
     }

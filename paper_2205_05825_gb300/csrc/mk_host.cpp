@@ -160,6 +160,8 @@ void free_device(mk_ctx *c) {
     cudaFree(c->d_bk);
     cudaFree(c->d_keyA);
     cudaFree(c->d_ks);
+    cudaFree(c->d_warp);
+    c->d_warp = nullptr;
     cudaFree(c->d_ksp);
     c->d_ksp = nullptr;
     cudaFree(c->d_status);
@@ -278,8 +280,11 @@ int ensure_device_keys(mk_ctx *c) {
     std::vector<uint64_t> h_bk(bk_entries * N), h_keyA(keyA_entries * N);
     // The largest twiddle tables of the forms: NTT2's [2][N] uint4 plus the
     // per-prime tables [2 directions][2 primes][N] uint2 of the split kernel.
-    // After them, at N = 1024, the tables of the warp kernel.
-    std::vector<unsigned char> h_tw(4 * (size_t)N * 16 + (N == 1024 ? kWarpTableBytes : 0));
+    // The warp kernel's tables (N = 1024) have a buffer of their own: behind these they moved the buffers after them,
+    // and the kernels that read twiddles and public keys through L1 lost 2 to 8 % (one wave of variant 6 11.4 -> 12.1
+    // ms, of variant 3 8.2 -> 8.5 at k = 2, n = 140).
+    std::vector<unsigned char> h_tw(4 * (size_t)N * 16);
+    std::vector<unsigned char> h_warp(c->form == MK_FORM_NTT2 && N == 1024 ? kWarpTableBytes : 0);
     // src polynomial of BK entry e and of keyA entry r (negated for the CRS)
     auto bk_src = [&](size_t e) {
         const uint32_t i = (uint32_t)(e / ((size_t)n * 3 * d));
@@ -343,7 +348,7 @@ int ensure_device_keys(mk_ctx *c) {
             sp[2 * (2 * (size_t)N + m)] = i1, sp[2 * (2 * (size_t)N + m) + 1] = comp(i1, kP1);
             sp[2 * (3 * (size_t)N + m)] = i2, sp[2 * (3 * (size_t)N + m) + 1] = comp(i2, kP2);
         }
-        if (N == 1024) warp_tables(c->ntt_p1, c->ntt_p2, h_tw.data() + 4 * (size_t)N * 16);
+        if (!h_warp.empty()) warp_tables(c->ntt_p1, c->ntt_p2, h_warp.data());
         auto dual = [&](const uint32_t *src, uint64_t *dst, bool negate) {
             std::vector<uint32_t> r1(N), r2(N);
             c->ntt_p1.to_device(src, r1.data(), negate);
@@ -394,6 +399,7 @@ int ensure_device_keys(mk_ctx *c) {
     if (!c->d_bk) MK_CUDA(c, cudaMalloc(&c->d_bk, h_bk.size() * 8));
     if (!c->d_keyA) MK_CUDA(c, cudaMalloc(&c->d_keyA, h_keyA.size() * 8));
     if (!c->d_ks) MK_CUDA(c, cudaMalloc(&c->d_ks, (size_t)k * c->ks_words() * 4));
+    if (!c->d_warp && !h_warp.empty()) MK_CUDA(c, cudaMalloc(&c->d_warp, h_warp.size()));
     if (!c->d_status) {
         MK_CUDA(c, cudaMalloc(&c->d_status, 16));
         MK_CUDA(c, cudaMemset(c->d_status, 0, 16));
@@ -406,6 +412,7 @@ int ensure_device_keys(mk_ctx *c) {
     // Work already enqueued may still read the previous keys.
     MK_CUDA(c, cudaStreamSynchronize(c->stream));
     MK_CUDA(c, cudaMemcpy(c->d_tw, h_tw.data(), h_tw.size(), cudaMemcpyHostToDevice));
+    if (!h_warp.empty()) MK_CUDA(c, cudaMemcpy(c->d_warp, h_warp.data(), h_warp.size(), cudaMemcpyHostToDevice));
     const size_t coef_bytes = c->form == MK_FORM_TC ? 4 : 8;
     MK_CUDA(c, cudaMemcpy(c->d_bk, h_bk.data(), h_bk.size() * coef_bytes, cudaMemcpyHostToDevice));
     MK_CUDA(c, cudaMemcpy(c->d_keyA, h_keyA.data(), h_keyA.size() * coef_bytes, cudaMemcpyHostToDevice));
