@@ -357,14 +357,7 @@ bootstrap_shared_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict_
         }
         __syncthreads();
     }
-    // no product is in flight when TMEM is freed; the exchange buffers are free since the last __syncthreads
-    if (warp == 0 && elect_one()) products_drain(st_smem_addr(ex), K.status);
-    __syncwarp();
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (threadIdx.x < 32)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem0), "r"(columns) : "memory");
+    release_tmem<columns, (size_t)Operands<3>::units * 16 + offsetof(SharedCtl, tmem), true>(K.status);
 }
 
 }  // namespace br

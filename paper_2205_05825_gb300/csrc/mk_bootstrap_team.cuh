@@ -68,16 +68,6 @@ __host__ __device__ inline TeamLayout team_layout(uint32_t k, uint32_t n, uint32
     return L;
 }
 
-// One lane of the warp (the compiler keeps the uniform registers that the
-// matrix instructions take their operands from in such a branch: the issue of
-// a step's products is on the critical path here, one gate 6.75 -> 6.57 ms; the
-// warp kernel, where it is not, measured slower with it).
-__device__ __forceinline__ bool elect_one() {
-    uint32_t r;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
-    return r != 0;
-}
-
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 
@@ -361,15 +351,7 @@ bootstrap_team_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
             }
         }
     }
-    // no product is in flight when TMEM is freed; a team's exchange buffer is free since its last quad_sync
-    if (warp == 0 && elect_one()) products_drain(st_smem_addr(ex), K.status);
-    __syncwarp();
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (threadIdx.x < 32)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem0), "r"(columns) : "memory");
-    __syncwarp();
+    release_tmem<columns, (size_t)Operands<T>::units * 16 + offsetof(WarpCtl, tmem), true>(K.status);
     cluster_arrive();  // no CTA leaves while another could still store into its shared memory
     cluster_wait();
 }

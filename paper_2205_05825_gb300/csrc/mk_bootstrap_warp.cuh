@@ -54,6 +54,8 @@
 // ciphertexts (hybrid product as in mk_bootstrap.cuh; arXiv 2205.05825,
 // Sec. 3.2 and 4.1).
 #pragma once
+#include <cstddef>
+
 #include <cuda_fp16.h>
 
 #include "mk_bootstrap.cuh"
@@ -321,24 +323,57 @@ __device__ __noinline__ void products_wait(uint32_t bar, uint32_t parity, volati
     atomicOr(status, kStatusWarp);
 }
 
-// At a kernel's end, the thread that issued a gate's products: every one of
-// them has completed when this returns, so that TMEM and shared memory can be
-// given back.  After a wait that ran out nothing else says so: later waits
-// return at once, and a barrier that missed a commit is a phase behind.  The
-// bound is this function's own.  bar: eight bytes of shared memory that
-// nothing else uses any more.
+// One lane of the warp (the compiler keeps the uniform registers that the
+// matrix instructions take their operands from in such a branch: the issue of
+// a step's products is on the critical path in the team kernel, one gate 6.75
+// -> 6.57 ms; the warp kernel, where it is not, measured slower with it).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+    return r != 0;
+}
+
+// The end of a CTA, by all its threads: waits for every product that its
+// threads have issued and gives TMEM back.  After a wait that ran out nothing
+// else says that they have completed: later waits return at once, and a barrier
+// that missed a commit is a phase behind.  The thread that issued a gate's (a
+// team's) products commits them to an mbarrier in the tables' first bytes, which
+// are free once all have arrived, and waits with a bound of its own.  ELECT:
+// that thread is the first warp's elected lane, else its lane 0.  TMEM_AT: where
+// in shared memory the address of the CTA's COLUMNS columns lies.  Not inlined,
+// and with one argument: in the kernels' own code the same lines changed the
+// register allocation of their loops (4096 gates at k = 2 1.5 to 7 % slower, 96
+// at k = 8 1.7 %).
 constexpr uint64_t kDrainNs = 1000000000ull;
-__device__ __noinline__ void products_drain(uint32_t bar, uint32_t *status) {
-    st_mbar_init(bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    st_fence_proxy_async();
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
-    const uint64_t t0 = st_globaltimer();
-    for (uint32_t it = 0; it < (1u << 30); ++it) {
-        if (st_mbar_try(bar, 0)) return;
-        if (st_globaltimer() - t0 > kDrainNs) break;
+template <uint32_t COLUMNS, size_t TMEM_AT, bool ELECT>
+__device__ __noinline__ void release_tmem(uint32_t *status) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const uint32_t *tmem = reinterpret_cast<const uint32_t *>(smem + TMEM_AT);
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const bool first = ((threadIdx.x >> 5) & 3) == 0;
+    if (ELECT ? (first && elect_one()) : (threadIdx.x & 127) == 0) {
+        const uint32_t bar = st_smem_addr(smem) + 8 * (threadIdx.x >> 7);
+        st_mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        st_fence_proxy_async();
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+        const uint64_t t0 = st_globaltimer();
+        bool done = false;
+        for (uint32_t it = 0; it < (1u << 30) && !done; ++it) {
+            done = st_mbar_try(bar, 0);
+            if (!done && st_globaltimer() - t0 > kDrainNs) break;
+        }
+        if (!done) atomicOr(status, kStatusWarp);
     }
-    atomicOr(status, kStatusWarp);
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(*tmem), "r"(COLUMNS) : "memory");
+    __syncwarp();
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&r)[16]) {
@@ -848,14 +883,8 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
         }
         quad_sync(bar);
     }
-    // no product is in flight when TMEM is freed; the slot's exchange buffer is free since its last quad_sync
-    if (warp == 0 && lane == 0) products_drain(st_smem_addr(ex), K.status);
-    __syncwarp();
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (threadIdx.x < 32)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(ctl->tmem), "r"(columns) : "memory");
+    constexpr size_t tmem_at = (size_t)Operands<kWarpMaxGates>::units * 16 + offsetof(WarpCtl, tmem);
+    release_tmem<columns, tmem_at, false>(K.status);
 }
 
 }  // namespace br
