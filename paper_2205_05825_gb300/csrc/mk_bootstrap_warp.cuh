@@ -646,6 +646,10 @@ __device__ __forceinline__ uint32_t word_of(const uint4 &a, int h) {
     return h == 0 ? a.x : (h == 1 ? a.y : (h == 2 ? a.z : a.w));
 }
 
+// HOOK: the instance that withholds a step's products (LaunchShape's
+// skip_key_step); the comparison in the loop costs the other one 2.8 % (4096
+// gates at k = 2).
+template <bool HOOK>
 __global__ void __launch_bounds__(128 * kWarpMaxGates, 1)
 bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ desc,
                       const uint32_t *__restrict__ ct_a, const uint32_t *__restrict__ ct_b,
@@ -767,7 +771,7 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
         for (int step = next_step(0); step < limit; step = next) {
             const int i = step / n + 1;
             const uint32_t e = abar[step];
-            const bool issue = step != S.skip_key_step;
+            const bool issue = !HOOK || step != S.skip_key_step;
             next = next_step(step + 1);
             const uint4 *bk = bk_all + (size_t)step * 9 * POLY + pr * (POLY / 2);
             uint32_t V[16];
@@ -794,7 +798,7 @@ bootstrap_warp_kernel(LaunchShape S, DeviceKeys K, const GateDesc *__restrict__ 
                 // the next slot's products run under this one's butterflies
                 if (s < k || (s == k + 1 && started)) {
                     cut_digits(s < k ? poly_of(s + 1, i) : poly_of(0, i), s < k ? e : abar[next]);
-                    start_products(s < k ? issue : next != S.skip_key_step);
+                    start_products(s < k ? issue : !HOOK || next != S.skip_key_step);
                 }
                 // R1 = <x, key1>, R2 = <x, key2> in place of x[0], x[1]: (d, A_jj), or (f0, f1) of v's digits
                 const uint4 *k1 = bk + (s <= k ? 0 : 3 * POLY);

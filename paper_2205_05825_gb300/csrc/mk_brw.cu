@@ -33,7 +33,7 @@ cudaError_t launch_bootstrap_warp(const LaunchShape &S, const DeviceKeys &K, con
     if (e != cudaSuccess) return e;
     const uint32_t g = warp_gates(S.k, S.n, count, (uint32_t)sms);
     const size_t smem = br::warp_layout(S.k, S.n, g).total;
-    auto kern = br::bootstrap_warp_kernel;
+    auto kern = S.skip_key_step < 0 ? br::bootstrap_warp_kernel<false> : br::bootstrap_warp_kernel<true>;
     e = br::allow_smem(kern);
     if (e != cudaSuccess) return e;
     const uint32_t grid = count < (uint32_t)sms ? count : (uint32_t)sms;
