@@ -123,7 +123,8 @@ template <int LOGN>
 __device__ __forceinline__ void mac_plane(uint32_t (&A)[8], const uint32_t (&x)[8], const uint32_t *__restrict__ plane,
                                           int tid, const PrimeOne &P) {
     const uint4 *s4 = reinterpret_cast<const uint4 *>(plane);
-    const uint4 a = __ldg(s4 + plane_unit_pos<LOGN>(2 * tid)), b = __ldg(s4 + plane_unit_pos<LOGN>(2 * tid + 1));
+    const int pos = plane_unit_pos<LOGN>(2 * tid);
+    const uint4 a = __ldg(s4 + pos), b = __ldg(s4 + plane_unit_next<LOGN>(pos));
     const uint32_t kv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
     for (int c = 0; c < 8; ++c) A[c] = red2p(A[c] + montmul(x[c], kv[c], P.p, P.pinv), P.twop);
