@@ -131,6 +131,25 @@ int mk_ctx_set_batch(mk_ctx *ctx, uint32_t max_gates_per_launch);
 enum { MK_CLUSTER_AUTO = 0, MK_CLUSTER_OFF = 1, MK_CLUSTER_ON = 2 };
 int mk_ctx_set_cluster(mk_ctx *ctx, int mode);
 
+/* Which blind-rotation kernel a gate call (or one chunk of mk_ctx_set_batch)
+ * of `count` gates gets with the context's present form, variant and cluster
+ * mode: kernels[0] (MK_BR_*) for its first gates[0] gates and, where it runs
+ * as two launches, kernels[1] for the other gates[1] (else 0 gates).  All give
+ * the same words; this is for tests and measurements.  MK_ESTATE until the
+ * keys are laid out on the device.  MK_BR_VARIANT: the kernel of the variant
+ * or of MK_FORM_FFT; MK_BR_TENSOR: MK_FORM_TC's launches.  No paper
+ * counterpart. */
+enum {
+    MK_BR_VARIANT = 0,
+    MK_BR_WARP = 1,
+    MK_BR_TEAM = 2,
+    MK_BR_SHARED = 3,
+    MK_BR_SMALL = 4,
+    MK_BR_CLUSTER = 5,
+    MK_BR_TENSOR = 6
+};
+int mk_ctx_get_route(mk_ctx *ctx, uint32_t count, uint32_t gates[2], int kernels[2]);
+
 /* Test hook for the kernels' bounded waits (no paper counterpart).  Every
  * wait of the staged blind rotation (variant 6) and of the cluster kernel for
  * a key copy, of MK_FORM_NTT2's kernels that compute on the tensor cores for

@@ -80,6 +80,8 @@ _SIGS = {
     "mk_gates_lin": (ctypes.c_int, [VP, VP, VP, VP, VP, ctypes.c_size_t]),
     "mk_gate_lin": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, VP]),
     "mk_debug_fault": (ctypes.c_int, [VP, ctypes.c_int, ctypes.c_int64, ctypes.c_uint64]),
+    "mk_ctx_get_route": (ctypes.c_int, [VP, ctypes.c_uint32, ctypes.POINTER(ctypes.c_uint32),
+                                        ctypes.POINTER(ctypes.c_int)]),
     "mk_ctx_set_circuit_exec": (ctypes.c_int, [VP, ctypes.c_int]),
     "mk_not": (ctypes.c_int, [VP, VP, VP, ctypes.c_size_t]),
     "mk_gates_noalloc": (ctypes.c_int, [VP, VP, VP, VP, VP, ctypes.c_size_t]),
@@ -245,6 +247,14 @@ class Context:
     def set_cluster(self, mode):
         """Latency (cluster) kernel: "auto" (small launches), "on" or "off"."""
         self._check(self.L.mk_ctx_set_cluster(self.h, CLUSTER_MODES[mode]), "mk_ctx_set_cluster")
+
+    KERNELS = ("variant", "warp", "team", "shared", "small", "cluster", "tensor")
+
+    def route(self, count):
+        """Blind-rotation launches of a call of `count` gates: [(gates, kernel name)], one or two."""
+        gates, kernels = (ctypes.c_uint32 * 2)(), (ctypes.c_int * 2)()
+        self._check(self.L.mk_ctx_get_route(self.h, count, gates, kernels), "mk_ctx_get_route")
+        return [(g, self.KERNELS[k]) for g, k in zip(gates, kernels) if g]
 
     FAULTS = {"none": 0, "skip_key_step": 1, "skip_digit_tile": 2, "skip_wire_ready": 3,
               "skip_key_tile": 4}

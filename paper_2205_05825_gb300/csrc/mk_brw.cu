@@ -159,6 +159,7 @@ uint32_t bootstrap_head(const LaunchShape &S, uint32_t count) {
 }
 
 bool team_form_chosen(const LaunchShape &S, uint32_t count) { return team_choice(S, count) >= 0; }
+bool shared_form_chosen(const LaunchShape &S, uint32_t count) { return team_choice(S, count) == 3; }
 
 cudaError_t launch_bootstrap_team(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc,
                                   const uint32_t *ct_a, const uint32_t *ct_b, const uint32_t *abar_in,

@@ -822,6 +822,21 @@ int mk_ctx_set_cluster(mk_ctx *c, int mode) {
     return MK_OK;
 }
 
+int mk_ctx_get_route(mk_ctx *c, uint32_t count, uint32_t gates[2], int kernels[2]) {
+    if (!c) return MK_EINVAL;
+    if (!gates || !kernels || count == 0) return fail(c, MK_EINVAL, "null pointer or no gates");
+    if (c->device < 0) return fail(c, MK_EDEVICE, "host-only context (device = -1)");
+    if (!c->dev_keys_valid) return fail(c, MK_ESTATE, "keys are not on the device yet");
+    MK_CUDA(c, cudaSetDevice(c->device));
+    const LaunchShape S = c->shape();
+    const uint32_t head = c->form == MK_FORM_TC ? 0 : bootstrap_head(S, count);
+    gates[0] = head ? head : count;
+    gates[1] = count - gates[0];
+    kernels[0] = blind_rotation_kernel(S, gates[0]);
+    kernels[1] = gates[1] ? blind_rotation_kernel(S, gates[1]) : kernels[0];
+    return MK_OK;
+}
+
 int mk_debug_fault(mk_ctx *c, int kind, int64_t arg, uint64_t wait_ns) {
     if (!c) return MK_EINVAL;
     if (kind != MK_FAULT_NONE && kind != MK_FAULT_SKIP_KEY_STEP && kind != MK_FAULT_SKIP_DIGIT_TILE &&

@@ -173,6 +173,9 @@ cudaError_t launch_bootstrap_team(const LaunchShape &S, const DeviceKeys &K, con
 // Whether launch_bootstrap_team takes a launch of `count` gates (its mode, and
 // under MK_CLUSTER_AUTO whether it is the faster form).
 bool team_form_chosen(const LaunchShape &S, uint32_t count);
+bool shared_form_chosen(const LaunchShape &S, uint32_t count);  // and whether that is the shared kernel
+// Which kernel (MK_BR_*) one launch of `count` gates gets.
+int blind_rotation_kernel(const LaunchShape &S, uint32_t count);
 uint32_t bootstrap_head(const LaunchShape &S, uint32_t count);
 
 // The two-prime form at N = 256, d = 3, bg_bit = 8 (mk_bootstrap_small.cuh):

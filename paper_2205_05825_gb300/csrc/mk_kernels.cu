@@ -400,6 +400,16 @@ BootstrapFn pick_cluster(const LaunchShape &S, uint32_t count) {
 }
 }  // namespace
 
+int blind_rotation_kernel(const LaunchShape &S, uint32_t count) {
+    if (S.form == MK_FORM_TC) return MK_BR_TENSOR;
+    BootstrapFn f = pick_cluster(S, count);
+    if (f == launch_bootstrap_team) return shared_form_chosen(S, count) ? MK_BR_SHARED : MK_BR_TEAM;
+    if (f && f != launch_bootstrap_small) return MK_BR_CLUSTER;
+    if (!f) f = pick(S);
+    if (f == launch_bootstrap_warp) return MK_BR_WARP;
+    return f == launch_bootstrap_small ? MK_BR_SMALL : MK_BR_VARIANT;
+}
+
 int cluster_capacity(const LaunchShape &S) {
     if (S.k + 1 > 8 || (S.form != MK_FORM_NTT && S.form != MK_FORM_NTT2)) return 0;
     if (S.logN == 8) return S.form == MK_FORM_NTT ? cluster_capacity_logn8_f0(S.k, S.n) : cluster_capacity_logn8_f1(S.k, S.n);
