@@ -137,7 +137,7 @@ class ClockSampler:
 
 
 # ----------------------------------------------------------------------------- roofline bookkeeping
-def work_per_cmux(P, form="ntt"):
+def work_per_cmux(P, form="ntt", warp=False):
     """Algorithmic work of one CMux step, in the unit of the form's ceiling.
     Tensor form: FLOPs of the dense products -- (2k+4) d Toeplitz products
     per step, each 4 byte planes x N^2 multiply-accumulates.
@@ -146,9 +146,19 @@ def work_per_cmux(P, form="ntt"):
     product, phase A and B), once per prime.  FFT form: FP64 instructions
     (an FMA counts one) -- 8 per complex butterfly, 4 per complex twist of
     each transformed point and 4 per pointwise complex multiply-add, on
-    M = N/2 folded points."""
+    M = N/2 folded points.
+    warp: the two-prime form's warp kernel, in butterflies' worth of the
+    multiply pipe and only what the method needs there, averaged over the
+    parties' steps: (k+5)/2 slots (the polynomials of parties not yet reached
+    are zero), each with d forward transforms' last four stages (the first six
+    are matrix products on the tensor cores), an inverse transform and 2 d N
+    products of three quarters of a butterfly each (three wide multiplies and
+    a Montgomery reduction per three products: 9 units of the pipe against a
+    butterfly's 4)."""
     k, d, N = P["k"], P["d"], P["N"]
     logn = N.bit_length() - 1
+    if warp:
+        return (k + 5) / 2 * 2 * ((4 * d + logn) * (N // 2) + 0.75 * 2 * d * N)
     if form == "tc":  # FLOPs (2 per multiply-accumulate) of the dense Toeplitz products, 4 byte planes
         return 2 * (2 * (k + 1) * d + 2 * d) * 4 * N * N
     if form == "fft":
@@ -175,10 +185,11 @@ def measured_peaks():
 
 
 def kernel_source_hash():
-    """Hash of the blind-rotation kernel's code with comments and whitespace
-    removed, so that an edit of its comments keeps a capture valid."""
+    """Hash of the blind-rotation kernel's code (its file and the ones it
+    includes) with comments and whitespace removed, so that an edit of its
+    comments keeps a capture valid."""
     h = hashlib.sha256()
-    for f in ("mk_bootstrap_warp.cuh",):
+    for f in ("mk_bootstrap_warp.cuh", "mk_bootstrap.cuh", "mk_bulk.cuh"):
         src = open(os.path.join(ROOT, "paper_2205_05825_gb300", "csrc", f), encoding="utf-8").read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
         src = re.sub(r"//[^\n]*", "", src)
@@ -558,8 +569,8 @@ def run_ours(args):
     total_ms = sum(step_ms)
     total_ms_max = reduce_max(total_ms, world)
     value = G * args.steps * world / (total_ms_max * 1e-3)
-    # per 4096 gates: descriptors, blind rotation, key-switch start values, key switch
-    launches_per_step = 4 * ((G + 4095) // 4096)
+    # per 4096 gates: descriptors, blind rotation (one or two), key-switch start values, key switch
+    launches_per_step = sum(3 + len(ctx.route(min(4096, G - at))) for at in range(0, G, 4096))
 
     # end to end through the public API with host buffers (pinned), copies inside
     h_types = torch.from_numpy(types.astype(np.uint8)).pin_memory()
@@ -643,7 +654,8 @@ def run_ours(args):
         plain4_ms = p0.elapsed_time(p1)
         plain4 = plain_g / (plain4_ms * 1e-3)
         ctx4.set_batch(4096)
-        work4 = work_per_cmux(P4, args.form) * P4["k"] * P4["n"]
+        warp4 = args.form == "ntt2" and v4 == 2
+        work4 = work_per_cmux(P4, args.form, warp4) * P4["k"] * P4["n"]
         ach4 = G4 * work4 / (br4_ms / max(br4_n, 1) * 1e-3) / scale
         k4 = {"gates_per_s": rate4, "gates": G4, "steps": len(ms4), "ms_per_batch": float(np.mean(ms4)),
               "latency_ms": {"p50": float(np.percentile(ms4, 50)), "p99": float(np.percentile(ms4, 99))},
@@ -652,7 +664,7 @@ def run_ours(args):
               "plain_one_gate_per_launch": {"gates_per_s": plain4, "gates": plain_g,
                                             "latency_ms": plain4_ms / plain_g, "batched_over_plain": rate4 / plain4},
               "roofline": {"bound": "tensor" if args.form == "tc" else "alu", "achieved": ach4, "peak": ceiling,
-                           "unit": UNIT_NAME[args.form], "frac": ach4 / ceiling,
+                           "unit": "G butterflies/s" if warp4 else UNIT_NAME[args.form], "frac": ach4 / ceiling,
                            "algorithmic_work_per_gate": work4, "br_share_of_step": br4_ms / sum(ms4)}}
         ctx4.close()
 
@@ -683,9 +695,9 @@ def run_ours(args):
 
     # roofline of the dominant kernel (blind rotation), live from the timed region
     avg_br_ms = br_ms / max(br_n, 1)
-    mm_per_gate = work_per_cmux(P, args.form) * P["k"] * P["n"]
+    warp = args.form == "ntt2" and variant == 2
+    mm_per_gate = work_per_cmux(P, args.form, warp) * P["k"] * P["n"]
     achieved = G * mm_per_gate / (avg_br_ms * 1e-3) / scale
-    warp = args.form == "ntt2" and variant == 2  # the warp kernel's: its first six forward stages are matrix products
     traffic_pg = ncu_traffic_per_gate() if warp else None
     if args.form == "tc":
         mp = measured_peaks()
@@ -700,7 +712,8 @@ def run_ours(args):
                     "frac_of_mma_sync_ceiling": achieved / ceiling,
                     "br_share_of_step": br_ms / total_ms if total_ms else None}
     else:
-        roofline = {"bound": "alu", "achieved": achieved, "peak": ceiling, "unit": UNIT_NAME[args.form],
+        roofline = {"bound": "alu", "achieved": achieved, "peak": ceiling,
+                    "unit": "G butterflies/s" if warp else UNIT_NAME[args.form],
                     "frac": achieved / ceiling, "traffic": (traffic_pg * G if traffic_pg is not None else None),
                     "kernel": ("bootstrap_warp_kernel (ntt2, N = 1024, variant 2)" if warp
                                else "bootstrap_ntt_kernel<%s, 10, variant %d>" % (args.form, variant)),
@@ -712,8 +725,9 @@ def run_ours(args):
                                        "fft": "complex FP64, 8 FP64 instructions per butterfly"}[args.form]),
                     "br_share_of_step": br_ms / total_ms if total_ms else None}
         if warp:
-            roofline["note"] = ("the forward transforms' first six stages run as exact matrix products on the tensor "
-                                "cores and are counted in the algorithmic work, so frac can pass 1")
+            roofline["note"] = ("work of the multiply pipe that the method needs, in butterflies: the last four forward "
+                                "stages (the first six are exact matrix products on the tensor cores), inverse "
+                                "transforms and products, of polynomials that are not identically zero")
 
     ctx.close()
     if rank != 0:

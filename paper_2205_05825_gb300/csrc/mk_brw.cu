@@ -100,7 +100,9 @@ cudaError_t launch_bootstrap_shared(const LaunchShape &S, const DeviceKeys &K, c
 }
 
 // The fastest kernel for this launch: the team kernel's teams a CTA, less one; 3: the shared kernel; -1: the warp
-// kernel.
+// kernel.  For the variants other than 2, -1 stands for their own kernel at the warp kernel's price, which is lower
+// (1.6 to 1.8 times at k = 2): the team kernel is never taken where their own is faster, and given up earlier than it
+// would have to be.
 int fastest(const LaunchShape &S, uint32_t count, uint32_t sms, double &cost) {
     int best = -1;
     cost = warp_cost(S, count, sms);

@@ -80,9 +80,10 @@ struct LaunchShape {
     // CTA (1, 2, 3), the gates resident at once (team_capacities).
     int cluster_mode;
     uint32_t team_cap[3];
-    // Bound on each wait of the staged kernel for a key copy, in ns of global
-    // time, and a test hook: the key copies of this CMux step are never
-    // issued, so the waits for them run out (-1: none).
+    // Bound on each wait of a kernel for its copies or matrix products, in ns
+    // of global time, and a test hook: the key copies (staged and cluster
+    // kernels) or products (warp, team and shared kernels) of this CMux step
+    // are never issued, so the waits for them run out (-1: none).
     uint64_t wait_ns;
     int64_t skip_key_step;
     // The same for the matrix-product key switch: this coefficient pair's key
@@ -284,6 +285,7 @@ cudaError_t launch_keyswitch(const LaunchShape &S, const DeviceKeys &K, const Ga
 bool keyswitch_tc_supported(const LaunchShape &S);
 size_t keyswitch_planes_bytes(const LaunchShape &S);  // 0 where it does not apply
 cudaError_t build_keyswitch_planes(const LaunchShape &S, const uint32_t *ks, void *planes, cudaStream_t st);
+// Refuses, before it writes, a count whose grid could not launch (2^31 blocks).
 cudaError_t launch_keyswitch_tc(const LaunchShape &S, const DeviceKeys &K, const GateDesc *desc, const uint32_t *ext,
                                 uint32_t *out, uint32_t count, cudaStream_t st);
 
