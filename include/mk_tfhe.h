@@ -186,8 +186,8 @@ int mk_debug_fault(mk_ctx *ctx, int kind, int64_t arg, uint64_t wait_ns);
 /* The k-bit operators evaluate their netlist level by level.  With graphs on
  * (the default) the level loop of each (operator, width, pairs) plan is
  * captured once as a CUDA graph on a stream the context owns and replayed on
- * the context's stream; it is captured again when the form, the variant or
- * the key buffers change.  Graphs are not used while timing is enabled
+ * the context's stream; it is captured again when the form, the variant, the
+ * cluster mode or the key buffers change.  Graphs are not used while timing is enabled
  * (mk_timing_enable) or with MK_FORM_TC.  No paper counterpart: launch
  * overhead only, results are identical either way. */
 int mk_ctx_set_graphs(mk_ctx *ctx, int on);
@@ -246,9 +246,10 @@ int mk_ctx_get_circuit_style(const mk_ctx *ctx, int *style);
  * `sample_gates` random ciphertexts on the context's device, keeps the
  * fastest for the context and stores it in *best (and, if ms_out is not
  * NULL, each variant's milliseconds in ms_out[0..MK_NUM_VARIANTS-1]).  It
- * synchronises the stream.  MK_FORM_FFT and MK_FORM_TC have one kernel for
- * every variant number: there it times nothing, reports 0 ms and keeps the
- * variant.  No paper counterpart: a tuning aid. */
+ * synchronises the stream.  MK_FORM_FFT has one kernel for every variant
+ * number: there it times nothing, reports 0 ms and keeps the variant.
+ * MK_FORM_TC has its two engines as variants 0 and 1 and reports 0 ms for
+ * the other numbers.  No paper counterpart: a tuning aid. */
 #define MK_NUM_VARIANTS 9
 int mk_ctx_set_variant(mk_ctx *ctx, int variant);
 int mk_ctx_get_variant(const mk_ctx *ctx, int *variant);

@@ -24,7 +24,7 @@
 // gates on the chip at once.  Measured (GB300, blind rotation of one wave):
 // k = 2: 1 gate 6.4 ms (the cluster kernel it replaces 11.5, the warp kernel
 // 15.7), 37 gates 7.7, 76 gates (T = 2) 8.4, 152 gates (T = 3) 10.7 against 14.3;
-// k = 4: 1 gate 13.3 (23.7), 5 gates 13.5; k = 8: 1 gate 34 ms against 150.
+// k = 4: 1 gate 13.2 (23.7), 5 gates 13.5; k = 8: 1 gate 34.5 ms against 150.
 // From about 77 gates the shared kernel (mk_bootstrap_shared.cuh) is faster.
 // A step is a chain of dependent phases: at T = 1 about 11.8 k clocks, of them
 // digits 0.6, two products 0.8 each, two sets of butterflies and key products
@@ -387,7 +387,7 @@ uint32_t team_registers() {
 // for its cluster: two clusters, each holding an SM's columns that the other
 // asks for, would wait for ever, and occupancy queries know nothing of TMEM.
 // T = 1 (256 columns) may have two CTAs an SM, T = 2 and 3 (512) must be alone
-// among them.  Registers see to it (255, 238 and 168 a thread of 65536); they
+// among them.  Registers see to it (255, 236 and 168 a thread of 65536); they
 // are the compiler's choice, so they are checked.  (Kernels without clusters
 // only delay each other: whoever holds columns gets to its end.)
 inline bool teams_fit_tmem() {

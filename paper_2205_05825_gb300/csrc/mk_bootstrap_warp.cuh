@@ -6,7 +6,7 @@
 // 8 elements a thread need three shared-memory exchanges with CTA barriers
 // per transform, and the multiplies of its butterflies (Shoup: one high and
 // two low multiplies, 8 cycles of a scheduler's 16-lane multiply pipe per
-// warp) bound it from below at about 13 k clocks per CMux step of a gate at
+// warp) bound it from below at about 12.5 k clocks per CMux step of a gate at
 // k = 2.  Here
 //  * coefficient m is u[c + 16 s], 16 columns x 64 rows.  Reducing a
 //    polynomial modulo the 64 factors X^16 - zeta_y of X^1024 + 1 mod p (the
