@@ -540,6 +540,9 @@ int get_plan(mk_ctx *c, int op, uint32_t k, uint32_t pairs, CircuitPlan **out) {
     plan->levels = L;
     MK_CUDA(c, cudaMemcpy(plan->d_desc, desc.data(), desc.size() * sizeof(GateDesc), cudaMemcpyHostToDevice));
     MK_CUDA(c, cudaMemcpy(plan->d_outs, outs.data(), outs.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    // A device memset, and a copy from pageable memory, may return before it is done; the context's stream need not
+    // wait for the legacy stream.
+    MK_CUDA(c, cudaStreamSynchronize(cudaStreamLegacy));
     *out = plan.get();
     c->plans[key] = std::move(plan);
     return MK_OK;
@@ -1016,6 +1019,7 @@ int mk_sync(mk_ctx *c) {
         MK_CUDA(c, cudaMemcpy(&st, c->d_status, sizeof(st), cudaMemcpyDeviceToHost));
         if (st) {
             MK_CUDA(c, cudaMemset(c->d_status, 0, sizeof(st)));
+            MK_CUDA(c, cudaStreamSynchronize(cudaStreamLegacy));  // or it could clear the next launch's
             if (st & kStatusStaged)
                 return fail(c, MK_ETIMEOUT, "a bounded wait of the staged blind rotation for a key copy gave up");
             if (st & kStatusKeyswitch)

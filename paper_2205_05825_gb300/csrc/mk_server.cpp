@@ -122,6 +122,7 @@ int server_plan(mk_server *s, int op, uint32_t k, uint32_t pairs, ServerPlan **o
     for (const Wire &w : net.outputs) outs.push_back(w.w * 2 + w.neg);
     MK_CUDA(c, cudaMalloc(&plan->d_outs, outs.size() * sizeof(int32_t)));
     MK_CUDA(c, cudaMemcpy(plan->d_outs, outs.data(), outs.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    MK_CUDA(c, cudaStreamSynchronize(cudaStreamLegacy));  // it may return before it is done
     *out = plan.get();
     s->plans[key] = std::move(plan);
     return MK_OK;
