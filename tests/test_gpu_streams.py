@@ -43,6 +43,7 @@ def test_first_calls_on_a_non_blocking_stream():
         while not server.step():
             pass
         other.sync()
+        server.close()
         for c in (plain, other):
             c.set_circuit_style("array")
         assert torch.equal(got, want) and torch.equal(again, want_s) and torch.equal(served, want_s)
